@@ -75,7 +75,48 @@ struct HostTables {
   std::vector<int32_t> gbase;   // first group of order (c, class); one extra end entry
   std::vector<int32_t> scnt;    // [N = 0..n][w < sc_w][m < sc_m]
   int sc_w = 1, sc_m = 1;
+  // the head of every order as prefix slot + last ranks (DevOrder::e4)
+  std::vector<uint32_t> e4;
+  std::vector<uint2> slots;
+  std::vector<int2> zones;
+  int e4_stride = 0;
 };
+
+// One zone of an order's compact form: entries from `q` on as a prefix slot
+// and the last `ranks` ranks, slots assigned in order of first use, until
+// another slot would be needed, a prefix would not fit its descriptor, or the
+// entries kept end.  The zone stops at a whole chunk.  Returns its end.
+int compact_zone(const uint4 *ent, int q, int count, int n, int ranks, int max_slots, uint2 *slots,
+                 std::vector<uint32_t> &out) {
+  // open-addressed table of the slots in use, keyed by their descriptor
+  int table[256];
+  std::fill(table, table + 256, -1);
+  int used = 0;
+  const int start = q;
+  for (; q < count; q++) {
+    uint8_t b[16];
+    std::memcpy(b, ent + q, 16);
+    const int w = b[0], rest = std::min(w, ranks), len = w - rest;
+    if (len > sg::FAST_PREFIX) break;
+    uint8_t d[8] = {(uint8_t)(len | (rest << 4)), 0, 0, 0, 0, 0, 0, 0};
+    for (int i = 0; i < len; i++) d[1 + i] = b[1 + i];
+    uint64_t key;
+    std::memcpy(&key, d, 8);
+    unsigned at = (unsigned)((key * 0x9E3779B97F4A7C15ull) >> 56);
+    while (table[at] >= 0 && std::memcmp(&slots[table[at]], d, 8) != 0) at = (at + 1) & 255;
+    if (table[at] < 0) {
+      if (used == max_slots) break;
+      std::memcpy(&slots[used], d, 8);
+      table[at] = used++;
+    }
+    uint32_t e = (uint32_t)table[at];
+    for (int i = 0; i < 3; i++) e |= (uint32_t)(i < rest ? b[1 + len + i] : n) << (8 + 8 * i);
+    out.push_back(e);
+  }
+  const int end = start + ((q - start) & ~31);
+  out.resize(out.size() - (size_t)(q - end));
+  return end;
+}
 
 // cnt[w][m] = number of w-subsets of {1..n} with sum m (saturating), w <= wlim
 struct SubsetCounts {
@@ -200,6 +241,24 @@ int build_tables(int n, int64_t cap, int c_max, bool even, HostTables &T) {
       T.count[(size_t)c * ncls + K] = (int32_t)(T.ent.size() - start);
     }
   }
+  // the compact forms of every order's head
+  const int orders = (c_max + 1) * ncls, per = sg::FAST_SLOTS2 + sg::FAST_SLOTS;
+  T.slots.assign((size_t)orders * per, make_uint2(0, 0));
+  T.zones.assign(orders, make_int2(0, 0));
+  std::vector<std::vector<uint32_t>> heads(orders);
+  int longest = 0;
+  for (int ti = 0; ti < orders; ti++) {
+    const uint4 *ent = &T.ent[T.base[ti]];
+    const int count = std::min(T.count[ti], sg::FAST_QUERIES);
+    int2 &z = T.zones[ti];
+    z.x = compact_zone(ent, 0, count, n, 2, sg::FAST_SLOTS2, &T.slots[(size_t)ti * per], heads[ti]);
+    z.y = compact_zone(ent, z.x, count, n, 3, sg::FAST_SLOTS, &T.slots[(size_t)ti * per + sg::FAST_SLOTS2], heads[ti]);
+    longest = std::max(longest, z.y);
+  }
+  T.e4_stride = longest + 64;  // padded: a chunk past the head is read ahead
+  T.e4.assign((size_t)orders * T.e4_stride, 0u);
+  for (int ti = 0; ti < orders; ti++)
+    std::copy(heads[ti].begin(), heads[ti].end(), T.e4.begin() + (size_t)ti * T.e4_stride);
   T.jmax = maxcost + 2;
   T.gbase.push_back((int32_t)T.grp.size());
   // scnt[N][w][m]: w-subsets of {1..N} with sum m (N = 0..n, w < sc_w, m <= the
@@ -229,7 +288,9 @@ int upload_tables(sogrand_code *c, const HostTables &T, int64_t cap) {
   const size_t bi = T.base.size() * sizeof(int32_t);
   const size_t bg = T.grp.size() * sizeof(uint2), bgb = T.gbase.size() * sizeof(int32_t);
   const size_t bs = T.scnt.size() * sizeof(int32_t);
-  const size_t bytes = al(be) + al(bc) + 2 * al(bi) + al(bg) + al(bgb) + al(bs);
+  const size_t b4 = T.e4.size() * sizeof(uint32_t), bsl = T.slots.size() * sizeof(uint2);
+  const size_t bz = T.zones.size() * sizeof(int2);
+  const size_t bytes = al(be) + al(bc) + 2 * al(bi) + al(bg) + al(bgb) + al(bs) + al(b4) + al(bsl) + al(bz);
   void *mem = nullptr;
   if (cudaMalloc(&mem, bytes) != cudaSuccess) return SOGRAND_ENOMEM;
   char *p = (char *)mem;
@@ -240,7 +301,13 @@ int upload_tables(sogrand_code *c, const HostTables &T, int64_t cap) {
   uint2 *dgrp = (uint2 *)(p + al(be) + al(bc) + 2 * al(bi));
   int32_t *dgbase = (int32_t *)((char *)dgrp + al(bg));
   int32_t *dscnt = (int32_t *)((char *)dgbase + al(bgb));
-  if (cudaMemcpy(dgrp, T.grp.data(), bg, cudaMemcpyHostToDevice) != cudaSuccess ||
+  uint32_t *de4 = (uint32_t *)((char *)dscnt + al(bs));
+  uint2 *dslots = (uint2 *)((char *)de4 + al(b4));
+  int2 *dzones = (int2 *)((char *)dslots + al(bsl));
+  if (cudaMemcpy(de4, T.e4.data(), b4, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(dslots, T.slots.data(), bsl, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(dzones, T.zones.data(), bz, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(dgrp, T.grp.data(), bg, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(dgbase, T.gbase.data(), bgb, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(dscnt, T.scnt.data(), bs, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(dent, T.ent.data(), be, cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -261,6 +328,10 @@ int upload_tables(sogrand_code *c, const HostTables &T, int64_t cap) {
   c->ord.count = dcount;
   c->ord.ncls = T.ncls;
   c->ord.class_size = T.class_size;
+  c->ord.e4 = de4;
+  c->ord.slots = dslots;
+  c->ord.zones = dzones;
+  c->ord.e4_stride = T.e4_stride;
   c->grp.grp = dgrp;
   c->grp.gbase = dgbase;
   c->grp.scnt = dscnt;

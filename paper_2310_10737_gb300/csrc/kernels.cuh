@@ -21,6 +21,18 @@ namespace sg {
 
 constexpr int TPB = 32 * WARPS_PER_BLOCK;
 
+// Resident blocks per SM that a schedule's kernels are compiled for.  Schedule
+// 8 takes 64 registers a thread; schedule 12 (its name: the second value of
+// sogrand_code_schedule) 48 registers, which is 10 blocks: at 40 (12 blocks)
+// the word's code spills and grows by 10%, and the two blocks more leave less
+// L1 (eBCH(64,57)^2, 20,000 frames: 27.0 ms at 10 blocks, 27.9 at 12).
+__host__ __device__ constexpr int resident_blocks(int minb) { return minb == 12 ? 10 : minb; }
+
+// The warp's index in its block, broadcast so that the compiler knows it to be
+// the same in every lane: the words' control flow is then provably uniform
+// and needs no divergence handling around its shuffles and votes.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(FULL, (int)(threadIdx.x >> 5), 0); }
+
 // dynamic shared memory of one block of a single-code kernel
 template <int NPL, class SYN>
 __host__ __device__ inline int block_scratch_bytes(int jmax) {
@@ -63,15 +75,17 @@ __device__ __forceinline__ void init_block_lock(unsigned char *tl, const SisoPar
 }
 
 // ---------------------------------------------------------------------------
-// LANES: the query order is enumerated by the lanes (DevCode::ord_lanes)
-// instead of read from the order table; a kernel of its own, so that the
-// table path's code and register allocation stay as they are.
-template <int NPL, class SYN, int MINB, bool LANES>
-__global__ void __launch_bounds__(TPB, MINB) k_decode(const DevCode code, const SisoParams P, const DecodeArgs a) {
+// MODE: where the query loop takes its patterns and whether the threshold rule
+// applies; kernels of their own, so that the code and register allocation of
+// each are not shaped by the others'.
+template <int NPL, class SYN, int MINB, int MODE>
+__global__ void __launch_bounds__(TPB, resident_blocks(MINB)) k_decode(const __grid_constant__ DevCode code,
+                                                      const __grid_constant__ SisoParams P,
+                                                      const __grid_constant__ DecodeArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   using LY = Layout<NPL, SYN>;
   constexpr int NM = (32 * NPL + 63) / 64;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   unsigned char *tl = block_tail(smem, LY::warp_bytes);
   init_block_lock(tl, P);
   Scratch<NPL, SYN> sc;
@@ -91,25 +105,20 @@ __global__ void __launch_bounds__(TPB, MINB) k_decode(const DevCode code, const 
       }
       lam[k] = x;
     }
-    float lapp[NPL];
     WordResult res;
-    int used_xf = 0;
-    siso_word<NPL, SYN, LANES>(code, P, sc, lam, lane, lapp, res, &used_xf);
-    const bool empty = res.nhit == 0;
-#pragma unroll
-    for (int k = 0; k < NPL; k++) {
+    siso_word<NPL, SYN, MODE>(code, P, sc, lam, lane, res, [&](int k, float x, float lapp, bool listed) {
       const int i = lane + 32 * k;
       if (i < n) {
-        if (a.llr_app) a.llr_app[base + i] = lapp[k];
-        if (a.llr_ext) a.llr_ext[base + i] = empty ? 0.f : __fsub_rn(lapp[k], sc.lam_at(i));
-        if (a.hard) a.hard[base + i] = lapp[k] < 0.f ? 1 : 0;
+        if (a.llr_app) a.llr_app[base + i] = lapp;
+        if (a.llr_ext) a.llr_ext[base + i] = listed ? __fsub_rn(lapp, x) : 0.f;
+        if (a.hard) a.hard[base + i] = lapp < 0.f ? 1 : 0;
       }
-    }
+    });
     if (lane == 0) {
       if (a.p_miss) a.p_miss[w] = res.pmiss;
       if (a.queries) a.queries[w] = res.queries;
       if (a.list_count) a.list_count[w] = res.nhit;
-      if ((used_xf & 1) && a.xf_count) atomicAdd(a.xf_count, 1);
+      if ((res.flags & 1) && a.xf_count) atomicAdd(a.xf_count, 1);
       if (a.wsum) atomicAdd(a.wsum, (unsigned long long)res.wsum);
     }
     if (a.list_words || a.list_app) {
@@ -177,17 +186,27 @@ __device__ __forceinline__ void tally_flush(const unsigned long long *slot, unsi
   if (xf_count && slot[1]) atomicAdd(xf_count, (int32_t)slot[1]);
 }
 
-// A word's context (frame, word, half, list index) is kept at the start of
-// the frame-check area sc.W(), which nothing else uses during a word (the
-// word's lambda follows it), and read back after the search: the registers
-// that held it are free while the search runs.
+// A word's context (frame, word, kind of half, list index) is kept at the
+// start of the frame-check area sc.W(), which nothing else uses during a word
+// (the word's lambda follows it), and read back after the search: the
+// registers that held it are free while the search runs.
 struct WordCtx {
-  int64_t f, li;
-  int32_t wd, half;
+  int32_t f, li, wd, rows;
 };
 static_assert(sizeof(WordCtx) <= 32, "the word's lambda follows the context in the frame-check area");
 
-// One component word of frame f in half `half` (rows when odd): lambda =
+// Offset of bit i of word wd in its frame of rows of nr bits: a row, a column
+// or (diag) a wrapped diagonal.
+__device__ __forceinline__ int bit_offset(int i, int wd, int nr, bool rows, bool diag) {
+  int r = rows ? wd : i;
+  if (diag && !rows) {
+    r = wd + i;
+    if (r >= nr) r -= nr;
+  }
+  return r * nr + ((rows || diag) ? i : wd);
+}
+
+// One component word of frame f (a row, or a column or diagonal): lambda =
 // L_Ch + fl32(alpha L_E) (L_A = 0 in the first half), SOGRAND, then L_E and
 // the hard decision of L_APP are stored and the query counters updated.
 // `code` is the code of this half's words (the row code in a row half, the
@@ -195,76 +214,61 @@ static_assert(sizeof(WordCtx) <= 32, "the word's lambda follows the context in t
 // and the second set of words may be wrapped diagonals (a.diag); otherwise
 // it is a square code.n x code.n frame with columns as the second set.
 // Returns the word's query count (-1: non-finite input).
-template <int NPL, class SYN, bool COHERENT, bool GEN, bool LANES = false>
+template <int NPL, class SYN, bool COHERENT, bool GEN, int MODE>
 __device__ __forceinline__ int product_word(const DevCode &code, const SisoParams &P, const ProductArgs &a,
-                                            const Scratch<NPL, SYN> &sc, int64_t f, int wd, int half, int lane) {
+                                            const Scratch<NPL, SYN> &sc, int f, int li, int wd, bool rows, bool first,
+                                            int lane) {
   constexpr int NM = (32 * NPL + 63) / 64;
 #ifdef SG_PHASE_PROFILE
   const long long t0 = clock64();
 #endif
-  const int n = code.n, nr = GEN ? a.nr : n;
-  const bool rows = (half & 1) != 0, diag = GEN && a.diag;
-  const size_t fb = (size_t)f * nr * (GEN ? a.nc : n);
+  const int n = code.n, nr = GEN ? a.nr : n, fsz = nr * (GEN ? a.nc : n);
+  const bool diag = GEN && a.diag;
   float lam[NPL];
-#pragma unroll
-  for (int k = 0; k < NPL; k++) {
-    const int i = lane + 32 * k;
-    float x = 0.f;
-    if (i < n) {
-      const size_t pos = fb + (rows ? (size_t)wd * nr + i
-                                    : (diag ? (size_t)((wd + i) % nr) * nr + i : (size_t)i * nr + wd));
-      x = __ldg(a.llr_ch + pos);
-      if (half > 1) x = __fadd_rn(x, __fmul_rn(a.alpha, ld_state<COHERENT>(a.le + pos)));  // L_A = alpha L_E
-    }
-    lam[k] = x;
-  }
-  float lapp[NPL];
-  WordResult res;
-  int used_xf = 0;
-  WordCtx *ctx = reinterpret_cast<WordCtx *>(sc.W());
-  if (lane == 0) {
-    ctx->f = f;
-    ctx->wd = wd;
-    ctx->half = half;
-  }
-  __syncwarp();
-  siso_word<NPL, SYN, LANES>(code, P, sc, lam, lane, lapp, res, &used_xf);
-  bool rows2;
   {
-    const volatile WordCtx *vc = ctx;
-    f = vc->f;
-    wd = vc->wd;
-    rows2 = (vc->half & 1) != 0;
-  }
-  const size_t fb2 = (size_t)f * nr * (GEN ? a.nc : n);
-  const bool empty = res.nhit == 0;
-  unsigned hb[NPL];
+    const size_t fb = (size_t)f * fsz;
+    const float *ch = a.llr_ch + fb, *le = a.le + fb;
+    float ext[NPL];
 #pragma unroll
-  for (int k = 0; k < NPL; k++) {
+    for (int k = 0; k < NPL; k++) {
+      const int i = lane + 32 * k;
+      lam[k] = ext[k] = 0.f;
+      if (i < n) {
+        const int pos = bit_offset(i, wd, nr, rows, diag);
+        lam[k] = __ldg(ch + pos);
+        if (!first) ext[k] = ld_state<COHERENT>(le + pos);
+      }
+    }
+    if (!first)  // L_A = alpha L_E
+#pragma unroll
+      for (int k = 0; k < NPL; k++) lam[k] = __fadd_rn(lam[k], __fmul_rn(a.alpha, ext[k]));
+  }
+  WordResult res;
+  if (lane == 0) *reinterpret_cast<int4 *>(sc.W()) = make_int4(f, li, wd, rows);
+  __syncwarp();
+  const volatile WordCtx *vc = reinterpret_cast<const volatile WordCtx *>(sc.W());
+  siso_word<NPL, SYN, MODE>(code, P, sc, lam, lane, res, [&](int k, float x, float lapp, bool listed) {
     const int i = lane + 32 * k;
-    if (i < n) {
-      const size_t pos = fb2 + (rows2 ? (size_t)wd * nr + i
-                                     : (diag ? (size_t)((wd + i) % nr) * nr + i : (size_t)i * nr + wd));
-      a.le[pos] = (empty || res.queries < 0) ? 0.f : __fsub_rn(lapp[k], sc.lam_at(i));
-    }
-    hb[k] = __ballot_sync(FULL, i < n && lapp[k] < 0.f);
-  }
+    if (i < n)
+      a.le[(size_t)vc->f * fsz + bit_offset(i, vc->wd, nr, vc->rows != 0, diag)] = listed ? __fsub_rn(lapp, x) : 0.f;
+    const unsigned hb = __ballot_sync(FULL, i < n && lapp < 0.f);
+    if (lane == 0) reinterpret_cast<unsigned *>(a.hb + ((size_t)vc->f * (GEN ? a.hbw : n) + vc->wd) * NM)[k] = hb;
+  });
+  f = vc->f;
+  wd = vc->wd;
   if (lane == 0) {
-    uint64_t *dst = a.hb + ((size_t)f * (GEN ? a.hbw : n) + wd) * NM;
-#pragma unroll
-    for (int wd2 = 0; wd2 < NM; wd2++) {
-      uint64_t v = hb[2 * wd2];
-      if (2 * wd2 + 1 < NPL) v |= (uint64_t)hb[2 * wd2 + 1] << 32;
-      dst[wd2] = v;
-    }
-    if (a.wq) a.wq[(size_t)f * (GEN ? a.hbw : n) + wd] = res.queries;
+    const size_t at = (size_t)f * (GEN ? a.hbw : n) + wd;
+    if (NPL & 1) reinterpret_cast<unsigned *>(a.hb + at * NM)[NPL] = 0u;  // the upper half of the last u64
+    if (a.wq) a.wq[at] = res.queries;
     if (res.queries >= 0) {
       atomicAdd(reinterpret_cast<unsigned long long *>(a.queries + f), (unsigned long long)res.queries);
       atomicMax(a.hmax + f, res.queries);
       sc.tally()[0] += (unsigned long long)res.wsum;
     }
-    sc.tally()[1] += used_xf & 1;
-    if ((used_xf & 2) && a.ctrl) atomicExch(a.ctrl + 3, 2);  // stops a persistent launch: reported as a timeout
+    if (res.flags) {
+      sc.tally()[1] += res.flags & 1;
+      if ((res.flags & 2) && a.ctrl) atomicExch(a.ctrl + 3, 2);  // stops a persistent launch: reported as a timeout
+    }
   }
   __syncwarp();
 #ifdef SG_PHASE_PROFILE
@@ -282,43 +286,58 @@ __device__ __forceinline__ int product_word(const DevCode &code, const SisoParam
 // iff parity(word & H_wc row t) = 0 for all t; every word of the other
 // orientation is a codeword of xc iff, for every t, the XOR of the words
 // selected by H_xc row t is zero (bit-sliced, no transpose).  Warp-uniform.
+//
+// The frame check and frame_finish run once per frame and half, after the
+// half's last word, on a warp whose SM is busy with words: they are kept short
+// (rolled loops, no per-bit divisions) because their code evicts the words'
+// from the instruction cache.
 template <int NPL>
 __device__ __forceinline__ bool frame_valid(const DevCode &wc, const DevCode &xc, const uint64_t *W, int lane) {
-  constexpr int NM = (32 * NPL + 63) / 64;
+  constexpr int NM = (32 * NPL + 63) / 64, W32 = 2 * NM;  // 32-bit words of a word, as stored (NPL of them used)
   const int nw = xc.n;  // words in W
-  bool ok = true;
+  const unsigned *Ws = reinterpret_cast<const unsigned *>(W);
+  unsigned own[NPL][NPL];  // [k]: this lane's words lane + 32 k
+  uint64_t hx[NPL];        // their columns in the code across
 #pragma unroll
   for (int k = 0; k < NPL; k++) {
     const int wd = lane + 32 * k;
-    if (wd < nw) {
-      for (int t = 0; t < wc.m && ok; t++) {
-        int p = 0;
+    hx[k] = wd < nw ? __ldg(xc.hcol + wd) : 0ull;
 #pragma unroll
-        for (int x = 0; x < NM; x++) p ^= __popcll(W[wd * NM + x] & __ldg(wc.hrow + t * NM + x));
-        if (p & 1) ok = false;
+    for (int j = 0; j < NPL; j++) own[k][j] = wd < nw ? Ws[wd * W32 + j] : 0u;
+  }
+  const unsigned *hrow = reinterpret_cast<const unsigned *>(wc.hrow);
+  unsigned bad = 0;
+#pragma unroll 1
+  for (int t0 = 0; t0 < wc.m; t0 += 32) {
+    unsigned row[NPL];  // lane t holds check t0 + t
+#pragma unroll
+    for (int j = 0; j < NPL; j++) row[j] = t0 + lane < wc.m ? __ldg(hrow + (t0 + lane) * W32 + j) : 0u;
+#pragma unroll 1
+    for (int t = 0; t < 32 && t0 + t < wc.m; t++) {
+      unsigned acc[NPL] = {};
+#pragma unroll
+      for (int j = 0; j < NPL; j++) {
+        const unsigned r = __shfl_sync(FULL, row[j], t);
+#pragma unroll
+        for (int k = 0; k < NPL; k++) acc[k] ^= own[k][j] & r;
       }
+#pragma unroll
+      for (int k = 0; k < NPL; k++) bad |= __popc(acc[k]) & 1;
     }
   }
-  ok = __all_sync(FULL, ok);
+  bool ok = !__any_sync(FULL, bad);
+#pragma unroll 1
   for (int t = 0; t < xc.m && ok; t++) {
-    uint64_t acc[NM];
+    unsigned acc[NPL] = {};
 #pragma unroll
-    for (int x = 0; x < NM; x++) acc[x] = 0;
+    for (int k = 0; k < NPL; k++)
+      if ((hx[k] >> t) & 1ull)
 #pragma unroll
-    for (int k = 0; k < NPL; k++) {
-      const int wd = lane + 32 * k;
-      if (wd < nw && ((__ldg(xc.hrow + t * NM + (wd >> 6)) >> (wd & 63)) & 1ull))
+        for (int j = 0; j < NPL; j++) acc[j] ^= own[k][j];
+    unsigned any = 0;
 #pragma unroll
-        for (int x = 0; x < NM; x++) acc[x] ^= W[wd * NM + x];
-    }
-    bool zero = true;
-#pragma unroll
-    for (int x = 0; x < NM; x++) {
-      const unsigned lo_ = __reduce_xor_sync(FULL, (unsigned)acc[x]);
-      const unsigned hi_ = __reduce_xor_sync(FULL, (unsigned)(acc[x] >> 32));
-      zero = zero && lo_ == 0 && hi_ == 0;
-    }
-    ok = ok && zero;
+    for (int j = 0; j < NPL; j++) any |= __reduce_xor_sync(FULL, acc[j]);
+    ok = any == 0;
   }
   return ok;
 }
@@ -337,6 +356,7 @@ __device__ __forceinline__ bool frame_valid_diag(const DevCode &code, const uint
   for (int k = 0; k < NPL; k++) {
     const int x = lane + 32 * k;
     if (x < n) {
+#pragma unroll 1
       for (int t = 0; t < code.m && ok; t++) {
         int p = 0;
 #pragma unroll
@@ -344,9 +364,12 @@ __device__ __forceinline__ bool frame_valid_diag(const DevCode &code, const uint
         if (p & 1) ok = false;
       }
       uint64_t syn = 0;
+      int w = x;  // (x + j) mod n after rows, (x - j) mod n after diagonals
+#pragma unroll 1
       for (int j = 0; j < n; j++) {
-        const int w = rows ? (x + j) % n : (x - j + n) % n;
         if ((W[w * NM + (j >> 6)] >> (j & 63)) & 1ull) syn ^= __ldg(code.hcol + j);
+        w += rows ? 1 : n - 1;
+        if (w >= n) w -= n;
       }
       if (syn) ok = false;
     }
@@ -358,24 +381,59 @@ __device__ __forceinline__ bool frame_valid_diag(const DevCode &code, const uint
 // words of the last half: rows (bit j of word i is bit (i, j)), columns
 // (bit i of word j is bit (i, j)) or, for a QC-GLDPC, wrapped diagonals (bit j
 // of word (i - j) mod n is bit (i, j)).
+// Columns are turned into rows first (a ballot collects one row of 32
+// columns), so a byte of the output is a shift of its row when rows start on
+// byte boundaries.
 template <int NPL>
 __device__ __forceinline__ void frame_finish(const ProductArgs &a, int64_t f, bool rows, int half, int status,
-                                             const uint64_t *W, int lane) {
-  constexpr int NM = (32 * NPL + 63) / 64;
-  const int nr = a.nr, nbits = a.nr * a.nc;
+                                             uint64_t *W, int lane) {
+  constexpr int NM = (32 * NPL + 63) / 64, W32 = 2 * NM;
+  const int nr = a.nr, nc = a.nc, nbits = nr * nc;
   const int nbytes = (nbits + 7) / 8;
   uint8_t *out = a.bits + (size_t)f * nbytes;
-  for (int by = lane; by < nbytes; by += 32) {
-    unsigned v = 0;
+  unsigned *Ws = reinterpret_cast<unsigned *>(W);
+  const bool diag = !rows && a.diag;
+  if (!rows && !diag) {
+    unsigned own[NPL][NPL];  // [k]: columns lane + 32 k
 #pragma unroll
-    for (int t = 0; t < 8; t++) {
-      const int p = by * 8 + t;
-      if (p < nbits) {
-        const int i = p / nr, j = p - i * nr;
-        const uint64_t word = rows     ? W[i * NM + (j >> 6)] >> (j & 63)
-                              : a.diag ? W[((i - j + nr) % nr) * NM + (j >> 6)] >> (j & 63)
-                                       : W[j * NM + (i >> 6)] >> (i & 63);
-        v |= (unsigned)(word & 1ull) << t;
+    for (int k = 0; k < NPL; k++)
+#pragma unroll
+      for (int j = 0; j < NPL; j++) own[k][j] = lane + 32 * k < nr ? Ws[(lane + 32 * k) * W32 + j] : 0u;
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < NPL; j++) {
+#pragma unroll 1
+      for (int i = 32 * j; i < 32 * j + 32 && i < nc; i++) {
+#pragma unroll
+        for (int k = 0; k < NPL; k++) {
+          const unsigned row = __ballot_sync(FULL, own[k][j] & 1u);
+          own[k][j] >>= 1;
+          if (lane == k) Ws[i * W32 + k] = row;
+        }
+      }
+    }
+    __syncwarp();
+  }
+  const bool aligned = (nr & 7) == 0 && !diag;
+#pragma unroll 1
+  for (int by = lane; by < nbytes; by += 32) {
+    int i = by * 8 / nr, j = by * 8 - i * nr;
+    unsigned v = 0;
+    if (aligned) {
+      v = Ws[i * W32 + (j >> 5)] >> (j & 31);
+    } else {
+#pragma unroll 1
+      for (int t = 0; t < 8 && i < nc; t++) {
+        int w = i;
+        if (diag) {
+          w = i - j;
+          if (w < 0) w += nr;
+        }
+        v |= ((Ws[w * W32 + (j >> 5)] >> (j & 31)) & 1u) << t;
+        if (++j == nr) {
+          j = 0;
+          i++;
+        }
       }
     }
     out[by] = (uint8_t)v;
@@ -388,29 +446,31 @@ __device__ __forceinline__ void frame_finish(const ProductArgs &a, int64_t f, bo
 }
 
 // ---- plain form: one launch per half iteration, then a check launch ----
-template <int NPL, class SYN, bool ROWS, int MINB, bool GEN>
-__global__ void __launch_bounds__(TPB, MINB) k_product_half(const DevCode rowc, const DevCode colc, const SisoParams P,
-                                                         const ProductArgs a, int half) {
+template <int NPL, class SYN, int MINB, bool GEN, int MODE>
+__global__ void __launch_bounds__(TPB, resident_blocks(MINB))
+    k_product_half(const __grid_constant__ DevCode rowc, const __grid_constant__ DevCode colc,
+                   const __grid_constant__ SisoParams P, const __grid_constant__ ProductArgs a, int half) {
   extern __shared__ __align__(16) unsigned char smem[];
   using LY = Layout<NPL, SYN>;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int jm = max(rowc.jmax, colc.jmax);
   unsigned char *tl = block_tail(smem, LY::warp_bytes);
   init_block_lock(tl, P);
   Scratch<NPL, SYN> sc;
   bind_scratch(sc, smem, warp, LY::warp_bytes, tl + TAIL_BYTES, tl);
-  const DevCode &code = ROWS ? rowc : colc;  // the code of this half's words
-  const int n = ROWS ? a.nc : a.nr;          // words per frame in this half
+  const bool rows = (half & 1) != 0;
+  const DevCode &code = GEN && !rows ? colc : rowc;  // the code of this half's words
+  const int n = rows ? a.nc : a.nr;                  // words per frame in this half
   const int64_t items = a.n_frames * n;
   const int64_t nwarps = (int64_t)gridDim.x * WARPS_PER_BLOCK;
   tally_clear(sc.tally(), lane);
   for (int64_t it = (int64_t)blockIdx.x * WARPS_PER_BLOCK + warp; it < items; it += nwarps) {
     const int64_t f = it / n;
-    const int wd = (int)(it - f * n);
+    int wd = (int)(it - f * n);
     const int32_t fs = __ldg(a.fstate + f);
     if (fs != F_RUN && fs != F_BAD_PENDING) continue;  // finished frames only: a flag raised during
                                                         // this half must not change which words run
-    const int q = product_word<NPL, SYN, false, GEN>(code, P, a, sc, f, wd, half, lane);
+    const int q = product_word<NPL, SYN, false, GEN, MODE>(code, P, a, sc, (int)f, 0, wd, rows, half == 1, lane);
     if (lane == 0 && q < 0) atomicExch(a.fstate + f, (int32_t)F_BAD_PENDING);
   }
   tally_flush(sc.tally(), a.wsum, a.xf_count, lane);
@@ -454,24 +514,16 @@ __global__ void __launch_bounds__(TPB) k_product_check(const DevCode rowc, const
 
 // ---- persistent forms: one launch decodes the whole batch ----
 
-// Draw a word ticket and wait until its slot of the frame-half list is
-// filled.  A filled slot holds +(e + 1) for an odd half of list entry e and
-// -(e + 1) for an even one: the slot itself says which half it is, so a
-// ticket that the half skips (codes of different lengths) is recognised even
-// after the frame has moved on to its next half.  Returns 1 with *f1 = the
-// signed slot value, or 0 when the list is done (every frame finished or
-// parked) or the launch's error word *err_w is set.  The wait backs off
-// exponentially and gives up after max_spin microseconds of sleep, setting
-// the error word.  All reads of shared state are made by lane 0 and
-// broadcast, so the whole warp takes the same branch.
 // Lane 0 of a warp publishes and observes the list with release/acquire
 // operations at GPU scope; __syncwarp orders the other lanes' accesses before
-// (release) or after (acquire) lane 0's, so no lane runs a full fence per
-// word (1-2% faster than a __threadfence on both sides).
-__device__ __forceinline__ int32_t ld_acquire_gpu(const volatile int32_t *p) {
+// (release) or after (acquire) lane 0's, so no lane runs a full fence.
+__device__ __forceinline__ int32_t ld_acquire_gpu(const int32_t *p) {
   int32_t v;
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ void st_release_gpu(int32_t *p, int32_t v) {
+  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ int32_t atom_add_acq_rel_gpu(int32_t *p, int32_t x) {
   int32_t old;
@@ -479,100 +531,101 @@ __device__ __forceinline__ int32_t atom_add_acq_rel_gpu(int32_t *p, int32_t x) {
   return old;
 }
 
-__device__ __forceinline__ int sched_take(int32_t *ctrl_w, int32_t *err_w, const volatile int32_t *queue,
-                                          int64_t nslots, int64_t frames, int slot_n, int max_spin, int lane,
-                                          int *slot_out, int *word_out, int *f1_out, int *waited) {
-  volatile int32_t *ctrl = ctrl_w;  // [0] slots reserved, [1] word tickets, [2] finished frames
-  const volatile int32_t *err = err_w;
+// A filled slot of the frame-half list holds +v for an odd half and -v for an
+// even one, v = 2 (list entry + 1) + 1 for a frame's first half and
+// 2 (list entry + 1) for a later one.  The slot itself says which kind of half
+// it is, so a ticket that the half skips (codes of different lengths) is
+// recognised even after the frame has moved on, and a word needs no look at
+// its frame's counters before it starts.
+__device__ __forceinline__ int32_t slot_value(int li, int half) {
+  const int v = 2 * (li + 1) + (half == 1);
+  return (half & 1) ? v : -v;
+}
+
+// Draw a word ticket and wait until its slot of the frame-half list is filled.
+// Returns the signed slot value, or 0 when the list is done (every frame
+// finished or parked) or the launch's error word a.ctrl[3] is set.  The wait
+// backs off exponentially and gives up after max_spin microseconds of sleep,
+// setting the error word.  All reads of shared state are made by lane 0 and
+// broadcast, so the whole warp takes the same branch.
+__device__ __forceinline__ int sched_take(const ProductArgs &a, int slot_n, int lane, int *word_out, int *waited) {
   int ticket = 0;
-  if (lane == 0) ticket = atomicAdd(ctrl_w + 1, 1);
+  if (lane == 0) ticket = atomicAdd(a.ctrl + 1, 1);
   ticket = __shfl_sync(FULL, ticket, 0);
   const int slot = ticket / slot_n;
-  int f1 = 0, st = 0;  // st: 0 wait, 1 work, 2 stop
-  long long slept = 0;
-  unsigned nap = 64;
+  *word_out = ticket - slot * slot_n;
+  const bool real = slot < a.n_frames * a.max_half;  // a frame has at most max_half halves
+  int v = 0;
+  unsigned slept = 0, nap = 64;  // slept: microseconds / 1.024
   for (;;) {
+    int stop = 0;
     if (lane == 0) {
-      if (*err != 0) {
-        st = 2;
-      } else if (slot < nslots && (f1 = ld_acquire_gpu(queue + slot)) != 0) {
-        st = 1;
-      } else if (ctrl[2] >= frames) {
-        st = 2;  // every frame finished: this ticket has no work
-      } else {
-        st = 0;
-      }
+      if (real) v = ld_acquire_gpu(a.queue + slot);
+      // an error, or every frame finished and this ticket has no work
+      const volatile int32_t *ctrl = a.ctrl;
+      if (ctrl[3] != 0)
+        stop = 1;
+      else if (v == 0)
+        stop = ctrl[2] >= a.n_frames;
     }
-    st = __shfl_sync(FULL, st, 0);
-    if (st != 0) break;
+    stop = __shfl_sync(FULL, stop, 0);
+    v = __shfl_sync(FULL, v, 0);
+    if (stop) return 0;
+    if (v != 0) break;
     *waited = 1;
-    if (slept > (long long)max_spin * 1000) {
-      if (lane == 0) atomicExch(err_w, 1);
-      st = 2;
-      break;
+    if ((slept >> 10) > (unsigned)a.max_spin) {
+      if (lane == 0) atomicExch(a.ctrl + 3, 1);
+      return 0;
     }
     __nanosleep(nap);
     slept += nap;
     if (nap < 8192) nap <<= 1;
   }
-  if (st == 2) return 0;
-  *slot_out = slot;
-  *word_out = ticket - slot * slot_n;
-  *f1_out = __shfl_sync(FULL, f1, 0);
   __syncwarp();  // after lane 0's acquire: the warp reads the frame's state for this half
-  return 1;
+  return v;
 }
 
-// After the last word of a half of frame f (list entry f + 1 in the launch's
-// index space `gf`): check the frame and finish it, park it (a serving epoch
-// ran out: its state stays for the next launch) or append its next half.
+// After the last word of a half of frame f (list entry li): check the frame
+// and finish it, park it (a serving epoch ran out: its state stays for the
+// next launch) or append its next half.  `words` is the shared address of the
+// warp's frame-check area.
 template <int NPL, bool GEN>
-__device__ __forceinline__ void frame_after_half(const DevCode &wc, const DevCode &xc, const ProductArgs &a,
-                                                 int32_t *ctrl, int32_t *queue_w, int64_t f, int64_t gf, int half,
-                                                 uint64_t *W, int lane) {
+__device__ __forceinline__ void frame_after_half(const DevCode &wc, const DevCode &xc, const ProductArgs &a, int f, int li,
+                                              unsigned words, int lane) {
   constexpr int NM = (32 * NPL + 63) / 64;
+  uint64_t *W = sptr<uint64_t>(words);
   const int n = xc.n;  // words of this half
   __syncwarp();  // after lane 0's acquire of the frame's word count: the other words' results
-  __threadfence();
-  const bool rows = (half & 1) != 0;
-  const int hbw = GEN ? a.hbw : n;
-  for (int x = lane; x < n * NM; x += 32) W[x] = ld_state<true>(a.hb + (size_t)f * hbw * NM + x);
+  const uint64_t *hb = a.hb + (size_t)f * (GEN ? a.hbw : n) * NM;
+#pragma unroll 1
+  for (int x = lane; x < n * NM; x += 32) W[x] = ld_state<true>(hb + x);
+  const int half = __ldcg(a.half_cur + f), bad = __ldcg(a.bad + f);
+  const int stop = a.half_stop ? __ldcg(a.half_stop + f) : a.max_half;
   __syncwarp();
+  const bool rows = (half & 1) != 0;
   const bool ok = (GEN && a.diag) ? frame_valid_diag<NPL>(wc, W, rows, lane) : frame_valid<NPL>(wc, xc, W, lane);
-  int bad = 0, stop = 0;
   if (lane == 0) {
-    bad = __ldcg(a.bad + f);
     a.par_queries[f] += __ldcg(a.hmax + f);
     a.hmax[f] = 0;
-    stop = a.half_stop ? __ldcg(a.half_stop + f) : a.max_half;
   }
-  bad = __shfl_sync(FULL, bad, 0);
-  stop = __shfl_sync(FULL, stop, 0);
   if (bad || ok || half >= a.max_half) {
     frame_finish<NPL>(a, f, rows, half, bad ? 2 : (ok ? 0 : 1), W, lane);
-    __threadfence();
-    if (lane == 0) atomicAdd(ctrl + 2, 1);
-  } else if (half >= stop) {
-    if (lane == 0) {  // parked: resumes at half + 1 in a later launch
-      a.half_cur[f] = half + 1;
-      a.done_words[f] = 0;
-      __threadfence();
-      atomicAdd(ctrl + 2, 1);
-    }
+    if (lane == 0) atomicAdd(a.ctrl + 2, 1);
   } else if (lane == 0) {
     a.half_cur[f] = half + 1;
     a.done_words[f] = 0;
-    __threadfence();
-    const int t = atomicAdd(ctrl + 0, 1);  // < nslots: every frame appends at most max_half - 1 times
-    const int e = (int)(gf + 1);
-    atomicExch(queue_w + t, ((half + 1) & 1) ? e : -e);  // the sign gives the half's parity
+    if (half >= stop) {  // parked: resumes at half + 1 in a later launch
+      atomicAdd(a.ctrl + 2, 1);
+    } else {
+      const int t = atomicAdd(a.ctrl + 0, 1);  // < nslots: every frame appends at most max_half - 1 times
+      st_release_gpu(a.queue + t, slot_value(li, half + 1));
+    }
   }
   __syncwarp();
 }
 
-// Frame-halves are appended to a list (a.queue[s] = +-(frame + 1) once slot s
-// is filled, negative for an even half); the first F slots hold every
-// frame's current half.  Warps draw global word tickets T: slot T / slot_n,
+// Frame-halves are appended to a list (a.queue, see slot_value); the first F
+// slots hold every frame's current half.  Warps draw global word tickets T: slot T / slot_n,
 // word T mod slot_n, one atomic per word.  The
 // warp that completes a frame's last word of a half runs the frame check and
 // either finishes the frame or appends it for its next half.  A warp whose
@@ -583,19 +636,19 @@ __device__ __forceinline__ void frame_after_half(const DevCode &wc, const DevCod
 // square product code whose words all use rowc, with no per-word selection
 // of a code (selecting one of two parameter structs at run time makes the
 // compiler copy it to local memory).
-template <int NPL, class SYN, int MINB, bool GEN, bool LANES = false>
-__global__ void __launch_bounds__(TPB, MINB) k_product_persistent(const DevCode rowc, const DevCode colc,
-                                                               const SisoParams P, const ProductArgs a) {
+template <int NPL, class SYN, int MINB, bool GEN, int MODE>
+__global__ void __launch_bounds__(TPB, resident_blocks(MINB))
+    k_product_persistent(const __grid_constant__ DevCode rowc, const __grid_constant__ DevCode colc,
+                         const __grid_constant__ SisoParams P, const __grid_constant__ ProductArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   using LY = Layout<NPL, SYN>;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int jm = max(rowc.jmax, colc.jmax);
   unsigned char *tl = block_tail(smem, LY::warp_bytes);
   init_block_lock(tl, P);
   Scratch<NPL, SYN> sc;
   bind_scratch(sc, smem, warp, LY::warp_bytes, block_dp_area(smem, LY::warp_bytes, a.dp_area, a.dp_stride), tl);
   const int slot_n = GEN ? max(a.nr, a.nc) : rowc.n;  // tickets per list slot: the most words in a half
-  const int64_t nslots = a.n_frames * (int64_t)a.max_half;  // a frame has at most max_half halves
   tally_clear(sc.tally(), lane);
   if (lane == 0) atomicAdd(a.ctrl + 4, 1);  // one more active warp
   int waited = 0;
@@ -623,36 +676,27 @@ __global__ void __launch_bounds__(TPB, MINB) k_product_persistent(const DevCode 
       asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       break;
     }
-    int slot, w, f1;
-    if (!sched_take(a.ctrl, a.ctrl + 3, a.queue, nslots, a.n_frames, slot_n, a.max_spin, lane, &slot, &w, &f1,
-                    &waited))
-      break;
-    const bool rows = f1 > 0;                      // the slot's half is odd: a row half
-    int64_t li = (int64_t)(f1 > 0 ? f1 : -f1) - 1;  // list index
+    int w;
+    const int v = sched_take(a, slot_n, lane, &w, &waited);
+    if (v == 0) break;
+    const bool rows = v > 0;  // the slot's half is odd: a row half
+    const int li = ((rows ? v : -v) >> 1) - 1;  // list index
     const DevCode &code = GEN ? (rows ? rowc : colc) : rowc, &xcode = GEN ? (rows ? colc : rowc) : rowc;
     const int n = xcode.n;  // words in this half
     // a ticket past this half's words (codes of different lengths); decided
     // from the slot, since the frame may already be in its next half
     if (GEN && w >= n) continue;
-    int64_t f = a.frame_list ? (int64_t)a.frame_list[li] : li;
-    int half = 0;  // the slot's half: the frame cannot leave it before this word is done
-    if (lane == 0) half = __ldcg(a.half_cur + f);
-    half = __shfl_sync(FULL, half, 0);
-    if (lane == 0) reinterpret_cast<WordCtx *>(sc.W())->li = li;
-    const int q = product_word<NPL, SYN, true, GEN, LANES>(code, P, a, sc, f, w, half, lane);
-    {
-      const volatile WordCtx *vc = reinterpret_cast<const volatile WordCtx *>(sc.W());
-      f = vc->f;
-      li = vc->li;
-      half = vc->half;
-    }
+    int f = a.frame_list ? a.frame_list[li] : li;
+    const int q = product_word<NPL, SYN, true, GEN, MODE>(code, P, a, sc, f, li, w, rows, rows && (v & 1), lane);
+    f = *reinterpret_cast<const volatile int *>(sc.W());
     if (lane == 0 && q < 0) atomicExch(a.bad + f, 1);
     __syncwarp();  // every lane's L_E and hard decision, then lane 0 releases them
     int done = 0;
     if (lane == 0) done = atom_add_acq_rel_gpu(a.done_words + f, 1);  // acquire: the frame's other words
     done = __shfl_sync(FULL, done, 0);
     if (done != n - 1) continue;
-    frame_after_half<NPL, GEN>(code, xcode, a, a.ctrl, a.queue, f, li, half, sc.W(), lane);
+    const int li2 = *(reinterpret_cast<const volatile int *>(sc.W()) + 1);
+    frame_after_half<NPL, GEN>(code, xcode, a, f, li2, sc.base + LY::o_w, lane);
   }
   tally_flush(sc.tally(), a.wsum, a.xf_count, lane);
 }
@@ -683,7 +727,7 @@ static __global__ void k_persistent_init(const ProductArgs a) {
       a.done_words[f] = 0;
       a.hmax[f] = 0;
       if (a.half_stop) a.half_stop[f] = a.half_cur[f] + a.epoch_halves - 1;
-      queue[i] = (a.half_cur[f] & 1) ? (int32_t)(i + 1) : -(int32_t)(i + 1);  // signed by the half's parity
+      queue[i] = slot_value((int)i, a.half_cur[f]);
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -739,9 +783,10 @@ template <int NPL, class SYN>
 cudaError_t launch_decode(const DevCode &code, const SisoParams &P, const DecodeArgs &a, cudaStream_t s) {
   if (a.n_words <= 0) return cudaSuccess;
   const int smem = block_scratch_bytes<NPL, SYN>(code.jmax);
-  const bool eight = launch_minb(code.minb, a.n_words) == 8, lanes = code.ord_lanes && P.thr <= 0.f;
-  auto kern = lanes ? (eight ? k_decode<NPL, SYN, 8, true> : k_decode<NPL, SYN, 12, true>)
-                    : (eight ? k_decode<NPL, SYN, 8, false> : k_decode<NPL, SYN, 12, false>);
+  const bool eight = launch_minb(code.minb, a.n_words) == 8, lanes = code.ord_lanes;
+  auto kern = P.thr > 0.f ? (eight ? k_decode<NPL, SYN, 8, MODE_THR> : k_decode<NPL, SYN, 12, MODE_THR>)
+              : lanes     ? (eight ? k_decode<NPL, SYN, 8, MODE_LANES> : k_decode<NPL, SYN, 12, MODE_LANES>)
+                          : (eight ? k_decode<NPL, SYN, 8, MODE_TABLE> : k_decode<NPL, SYN, 12, MODE_TABLE>);
   cudaError_t e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const int grid = grid_for(kern, smem, a.n_words);
@@ -766,17 +811,11 @@ cudaError_t launch_product_half(const DevCode &rowc, const DevCode &colc, const 
   const int smem = block_scratch_bytes<NPL, SYN>(std::max(rowc.jmax, colc.jmax));
   const int64_t items = a.n_frames * ((half & 1) ? a.nc : a.nr);
   const int minb = launch_minb(rowc.minb, items);
-  if (half & 1) {
-    auto kern = minb == 8 ? k_product_half<NPL, SYN, true, 8, GEN> : k_product_half<NPL, SYN, true, 12, GEN>;
-    cudaError_t e = set_smem(kern, smem);
-    if (e != cudaSuccess) return e;
-    kern<<<grid_for(kern, smem, items), TPB, smem, s>>>(rowc, colc, P, a, half);
-  } else {
-    auto kern = minb == 8 ? k_product_half<NPL, SYN, false, 8, GEN> : k_product_half<NPL, SYN, false, 12, GEN>;
-    cudaError_t e = set_smem(kern, smem);
-    if (e != cudaSuccess) return e;
-    kern<<<grid_for(kern, smem, items), TPB, smem, s>>>(rowc, colc, P, a, half);
-  }
+  auto kern = P.thr > 0.f ? (minb == 8 ? k_product_half<NPL, SYN, 8, GEN, MODE_THR> : k_product_half<NPL, SYN, 12, GEN, MODE_THR>)
+                          : (minb == 8 ? k_product_half<NPL, SYN, 8, GEN, MODE_TABLE> : k_product_half<NPL, SYN, 12, GEN, MODE_TABLE>);
+  cudaError_t e = set_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  kern<<<grid_for(kern, smem, items), TPB, smem, s>>>(rowc, colc, P, a, half);
   return cudaGetLastError();
 }
 
@@ -813,9 +852,11 @@ cudaError_t launch_product_persistent(const DevCode &rowc, const DevCode &colc, 
                              : block_scratch_bytes<NPL, SYN>(std::max(rowc.jmax, colc.jmax));
   const int64_t words = a.n_frames * std::max(a.nr, a.nc);  // the most words of one half
   // the lanes-enumerated order: the square geometry only (GEN reads the table)
-  const bool eight = launch_minb(rowc.minb, words) == 8, lanes = !GEN && rowc.ord_lanes && P.thr <= 0.f;
-  auto kern = lanes ? (eight ? k_product_persistent<NPL, SYN, 8, GEN, !GEN> : k_product_persistent<NPL, SYN, 12, GEN, !GEN>)
-                    : (eight ? k_product_persistent<NPL, SYN, 8, GEN> : k_product_persistent<NPL, SYN, 12, GEN>);
+  const bool eight = launch_minb(rowc.minb, words) == 8, lanes = !GEN && rowc.ord_lanes;
+  constexpr int ML = GEN ? MODE_TABLE : MODE_LANES;
+  auto kern = P.thr > 0.f ? (eight ? k_product_persistent<NPL, SYN, 8, GEN, MODE_THR> : k_product_persistent<NPL, SYN, 12, GEN, MODE_THR>)
+              : lanes     ? (eight ? k_product_persistent<NPL, SYN, 8, GEN, ML> : k_product_persistent<NPL, SYN, 12, GEN, ML>)
+                          : (eight ? k_product_persistent<NPL, SYN, 8, GEN, MODE_TABLE> : k_product_persistent<NPL, SYN, 12, GEN, MODE_TABLE>);
   e = set_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int occ = 0;

@@ -49,7 +49,7 @@ struct ProductArgs {
   int32_t *xf_count;
   unsigned long long *wsum;  // [1] += summed pattern weights of all queries (may be null)
   // persistent form only (scratch)
-  int32_t *queue;             // [F * max_half] frame-halves: frame + 1 once a slot is filled, else 0
+  int32_t *queue;             // [F * max_half] frame-halves: slot_value() once a slot is filled, else 0
   int32_t *half_cur;          // [F] current half iteration of each frame
   int32_t *done_words;        // [F] words of the current half completed
   int32_t *bad;               // [F] a non-finite input was seen

@@ -30,7 +30,21 @@ struct DevOrder {
   const int32_t *count;   // [(c_max+1) * ncls] entries stored for (c, class)
   int32_t ncls;           // 2 for an even code (class = parity of y), else 1
   int32_t class_size;     // patterns in one class (saturated): count == class_size means the whole class
+  // The head of every order again, a pattern as its prefix and its last ranks
+  // (see query_loop_plain): order (c, class) = ti owns e4[ti * e4_stride ...]
+  // and slots[ti * (FAST_SLOTS2 + FAST_SLOTS) ...].
+  const uint32_t *e4;     // byte 0: prefix slot; bytes 1..3: the last ranks (0-based; n where there is none)
+  const uint2 *slots;     // byte 0: prefix length | ranks after it << 4; bytes 1..7: the prefix's ranks
+  const int2 *zones;      // [ti] queries in two-rank form (slots 0..31) and, from there, in three-rank form up to .y
+  int32_t e4_stride;
 };
+
+// Prefix slots of the two-rank and the three-rank form, and the longest prefix.
+// In query order the first 32 prefixes reach about 1000 queries when the last
+// two ranks are split off, and 64 about 9000 when the last three are (c = 0;
+// further for c > 0, where heavy patterns come later).
+constexpr int FAST_SLOTS2 = 32, FAST_SLOTS = 64, FAST_PREFIX = 7;
+constexpr int FAST_QUERIES = 16384;  // most queries of an order kept in these forms
 
 // The same orders as groups, for lanes that enumerate their patterns instead
 // of reading DevOrder::ent (DevCode::ord_lanes): a group is the run of
@@ -74,8 +88,8 @@ struct WordResult {
   int32_t queries;       // -1: invalid input
   int32_t nhit;
   float pmiss;
-  float logD;            // log(sum of list masses + R phi), relative to p(0)
   int32_t wsum;          // sum of the Hamming weights of the queried patterns
+  int32_t flags;         // remaining mass: bit 0 extended range used, bit 1 its area could not be locked
 };
 
 }  // namespace sg

@@ -213,6 +213,12 @@ struct RankRec {
   SYN h;
   float t;
 };
+// |lambda| of one reliability rank and the bit it belongs to, read together
+// when a listed word is recorded
+struct RankBit {
+  float a;
+  int bit;
+};
 
 // Shared memory of a block: one area per warp (below), then a tail: the lock
 // word of the block's remaining-mass area with the lock's poll limit (16
@@ -227,27 +233,36 @@ template <int NPL, class SYN>
 struct Layout {
   static constexpr int NT = 32 * NPL;
   static constexpr int NM = (NT + 63) / 64;
-  static constexpr int o_l2 = 0;                                      // float[NT] |lambda| log2(e), by rank
-  static constexpr int o_al = o_l2 + 4 * NT;                          // float[NT] |lambda|, by rank
-  static constexpr int o_hr = o_al + 4 * NT;  // RankRec[NT + 1] H column + mass factor, by rank; [n] neutral
+  static constexpr int o_rb = 0;                                      // RankBit[NT] |lambda| and bit, by rank
+  static constexpr int o_hr = o_rb + 8 * NT;  // RankRec[NT + 1] H column + mass factor, by rank; [n] neutral
   static constexpr int o_cw = align16(o_hr + (int)sizeof(RankRec<SYN>) * (NT + 1));  // u64[LMAX][NM] listed codewords
   static constexpr int o_lp = o_cw + 8 * LMAX * NM;                   // float[LMAX] log p(z)/p(0)
   static constexpr int o_wl = o_lp + 4 * LMAX;                        // float[LMAX] APP of each listed word
-  static constexpr int o_perm = o_wl + 4 * LMAX;                      // u8[NT] rank -> bit
-  static constexpr int o_w = align16(o_perm + NT);                    // u64[NT][NM] words of a frame (check)
+  static constexpr int o_w = align16(o_wl + 4 * LMAX);                // u64[NT][NM] words of a frame (check)
   // During a word the frame-check area is free: its first 32 bytes hold the
   // word's context (product kernels) and then float[NT] the word's lambda.
   // (A separate area would cost 1 KB per block, which moved the shared-memory
   // carveout of the 8-block schedule up a step and shrank L1 by a quarter.)
   static constexpr int o_lam = o_w + 32;
-  static_assert(32 + 4 * NT + 4 * (NPL + 1) <= 8 * NT * NM, "lambda and the word head fit in the frame-check area");
-  static constexpr int o_pf = align16(o_w + 8 * NT * NM);             // uint4[32] the next chunk of order entries
-  static constexpr int warp_bytes = o_pf + 16 * 32;
+  static constexpr int HEAD = NPL + 4;  // words after lambda: see Scratch::headv
+  static_assert(32 + 4 * NT + 4 * HEAD <= 8 * NT * NM, "lambda and the word head fit in the frame-check area");
+  // Prefix records of the query loop (uint4[FAST_SLOTS]); or, where a chunk is
+  // tested from the 16-byte entries, uint4[32], the next chunk's entries.
+  static constexpr int o_pf = align16(o_w + 8 * NT * NM);
+  static constexpr int warp_bytes = o_pf + 16 * (sizeof(SYN) == 4 ? FAST_SLOTS : 32);
   // block area (sized for the 8-byte XF policy): sfac[NT+1], fu[NT+1], fb[NT+1], ek[J] (float), he[J], ho[J]
   static __host__ __device__ int dp_bytes(int jm) { return align16(24 * (NT + 1) + 20 * jm + 32); }
   // a block of WARPS_PER_BLOCK warps: their areas, the tail and the remaining-mass area
   static __host__ __device__ int block_bytes(int jm) { return WARPS_PER_BLOCK * warp_bytes + TAIL_BYTES + dp_bytes(jm); }
 };
+
+// A typed pointer to a shared-memory address.  The scratch is carried as 32-bit
+// shared addresses: a generic pointer handed to an out-of-line function is
+// read with generic loads and 64-bit address arithmetic.
+template <class T>
+__device__ __forceinline__ T *sptr(unsigned addr) {
+  return reinterpret_cast<T *>(__cvta_shared_to_generic((size_t)addr));
+}
 
 // A warp's view of the block's scratch: its own area, the block's tail
 // (lock word and tally slots, shared memory) and the block's remaining-mass
@@ -256,36 +271,37 @@ struct Layout {
 template <int NPL, class SYN>
 struct Scratch {
   using LY = Layout<NPL, SYN>;
-  unsigned char *base;  // this warp's area
-  unsigned char *dp;    // the block's remaining-mass area
-  unsigned char *tl;    // the block's tail: lock word and poll limit, then the warps' tally slots
+  unsigned base;      // this warp's area (shared address)
+  unsigned tl;        // the block's tail (shared address): lock word and poll limit, then the warps' tally slots
+  unsigned char *dp;  // the block's remaining-mass area
   __device__ void bind(unsigned char *warp_area, unsigned char *dp_area, unsigned char *tail_area) {
-    base = warp_area;
+    base = (unsigned)__cvta_generic_to_shared(warp_area);
     dp = dp_area;
-    tl = tail_area;
+    tl = (unsigned)__cvta_generic_to_shared(tail_area);
   }
-  __device__ float *l2() const { return reinterpret_cast<float *>(base + LY::o_l2); }
-  __device__ float *al() const { return reinterpret_cast<float *>(base + LY::o_al); }
-  __device__ RankRec<SYN> *hr() const { return reinterpret_cast<RankRec<SYN> *>(base + LY::o_hr); }
-  __device__ uint64_t *cw() const { return reinterpret_cast<uint64_t *>(base + LY::o_cw); }
-  __device__ float *lp() const { return reinterpret_cast<float *>(base + LY::o_lp); }
-  __device__ float *wl() const { return reinterpret_cast<float *>(base + LY::o_wl); }
-  __device__ uint8_t *perm() const { return base + LY::o_perm; }
-  __device__ uint4 *pf() const { return reinterpret_cast<uint4 *>(base + LY::o_pf); }
-  __device__ uint64_t *W() const { return reinterpret_cast<uint64_t *>(base + LY::o_w); }
+  __device__ RankBit *rb() const { return sptr<RankBit>(base + LY::o_rb); }
+  // |lambda| log2(e) of rank e
+  __device__ float l2(int e) const { return __fmul_rn(rb()[e].a, LOG2E_F); }
+  __device__ RankRec<SYN> *hr() const { return sptr<RankRec<SYN>>(base + LY::o_hr); }
+  __device__ uint64_t *cw() const { return sptr<uint64_t>(base + LY::o_cw); }
+  __device__ unsigned *cw32() const { return sptr<unsigned>(base + LY::o_cw); }
+  __device__ float *lp() const { return sptr<float>(base + LY::o_lp); }
+  __device__ float *wl() const { return sptr<float>(base + LY::o_wl); }
+  __device__ uint4 *pf() const { return sptr<uint4>(base + LY::o_pf); }
+  __device__ uint4 *prec() const { return sptr<uint4>(base + LY::o_pf); }
+  __device__ uint64_t *W() const { return sptr<uint64_t>(base + LY::o_w); }
   // lambda by bit, kept here during the search and read back (volatile) for
   // the soft output, so that it holds no registers while the search runs
-  __device__ float *lamv() const { return reinterpret_cast<float *>(base + LY::o_lam); }
-  __device__ float lam_at(int i) const { return *reinterpret_cast<const volatile float *>(base + LY::o_lam + 4 * i); }
-  // the word's hard decision words (NPL) and 1-line parameter, after lambda
-  __device__ unsigned *headv() const { return reinterpret_cast<unsigned *>(base + LY::o_lam + 4 * LY::NT); }
-  __device__ unsigned head_at(int k) const { return *reinterpret_cast<const volatile unsigned *>(base + LY::o_lam + 4 * LY::NT + 4 * k); }
+  __device__ float *lamv() const { return sptr<float>(base + LY::o_lam); }
+  __device__ float lam_at(int i) const { return *sptr<const volatile float>(base + LY::o_lam + 4 * i); }
+  // after lambda: the word's hard decision words (NPL) and 1-line parameter,
+  // then (threshold rule) whether the double-float class total is known and it
+  __device__ unsigned *headv() const { return sptr<unsigned>(base + LY::o_lam + 4 * LY::NT); }
+  __device__ unsigned head_at(int k) const { return *sptr<const volatile unsigned>(base + LY::o_lam + 4 * LY::NT + 4 * k); }
   __device__ unsigned char *tail() const { return dp; }
-  __device__ int *lock() const { return reinterpret_cast<int *>(tl); }
+  __device__ int *lock() const { return sptr<int>(tl); }
   // this warp's tally slot: [0] summed pattern weights, [1] extended-range words
-  __device__ unsigned long long *tally() const {
-    return reinterpret_cast<unsigned long long *>(tl + 16) + 2 * (threadIdx.x >> 5);
-  }
+  __device__ unsigned long long *tally() const { return sptr<unsigned long long>(tl + 16) + 2 * (threadIdx.x >> 5); }
 };
 
 // The block's remaining-mass area is taken by one warp at a time.  Its holder
@@ -321,47 +337,38 @@ __device__ __forceinline__ void dp_unlock(int *lock, bool held, int lane) {
 // ----------------------------------------------------------------------------
 // warp helpers
 // ----------------------------------------------------------------------------
-// Bitonic sort of the warp's 32 * NPL keys, ascending, lane l holding sorted
-// positions l NPL .. l NPL + NPL - 1 (blocked).  The exchanges at distance
-// j < NPL stay inside a lane's registers, so fewer stages need shuffles (15
-// of 21 for 64 keys, 15 of 28 for 128; 20 and 25 when lane l held positions
-// l, l + 32, ...: 1-3% faster per word, most for 128-bit codes).  The stages
-// run as loops rather than unrolled: the sort is straight-line work done once
-// per word, and its unrolled form (about 20 stages of shuffles) made the
-// kernel's code large enough that warps in other phases of their words
-// stalled on instruction fetch (measured 4-10% slower for codes of 64 and 128
-// bits).
+// Bitonic sort of the warp's 32 * NPL 32-bit keys, ascending, lane l holding
+// sorted positions l NPL .. l NPL + NPL - 1 (blocked: exchanges at distances
+// below NPL stay inside a lane's registers, 15 of 21 stages take shuffles for
+// 64 keys and 15 of 28 for 128).  Every merge starts by comparing position p
+// with p ^ (size - 1), so that the lower position always keeps the smaller
+// key: a stage is a shuffle, a minimum or maximum by one bit of the lane, and
+// no direction.  Unrolled: 64 keys take about 130 instructions, where 64-bit
+// keys sorted in loops with a direction took 600 of a word's 3000.
 template <int NPL>
-__device__ __forceinline__ void warp_bitonic_sort_blocked(uint64_t (&v)[NPL], int lane) {
+__device__ __forceinline__ void warp_sort_blocked(unsigned (&v)[NPL], int lane) {
   constexpr int N = 32 * NPL;
-#pragma unroll 1
+#pragma unroll
   for (int size = 2; size <= N; size <<= 1) {
-#pragma unroll 1
-    for (int j = size >> 1; j >= NPL; j >>= 1) {
-      const int lj = j / NPL;  // partner lane: lane ^ lj, same register
 #pragma unroll
-      for (int k = 0; k < NPL; k++) {
-        const uint64_t o = __shfl_xor_sync(FULL, v[k], lj);
-        const int p = lane * NPL + k;
-        const bool asc = (p & size) == 0;
-        const bool lower = (lane & lj) == 0;
-        v[k] = (lower == asc) ? (v[k] < o ? v[k] : o) : (v[k] < o ? o : v[k]);
-      }
-    }
-    if constexpr (NPL > 1) {
+    for (int j = size >> 1; j > 0; j >>= 1) {
+      const bool flip = j == (size >> 1);
+      if (j >= NPL) {  // partners in other lanes
+        const bool low = (lane & (j / NPL)) == 0;
+        unsigned o[NPL];
 #pragma unroll
-      for (int j = NPL / 2; j > 0; j >>= 1) {
-        if (j <= (size >> 1)) {
+        for (int k = 0; k < NPL; k++)
+          o[k] = flip ? __shfl_xor_sync(FULL, v[NPL - 1 - k], size / NPL - 1) : __shfl_xor_sync(FULL, v[k], j / NPL);
 #pragma unroll
-          for (int k = 0; k < NPL; k++) {
-            if ((k & j) == 0) {
-              const int kp = k | j;
-              const bool asc = ((lane * NPL + k) & size) == 0;
-              const uint64_t a = v[k], b = v[kp];
-              const bool sw = asc ? (a > b) : (a < b);
-              v[k] = sw ? b : a;
-              v[kp] = sw ? a : b;
-            }
+        for (int k = 0; k < NPL; k++) v[k] = low ? min(v[k], o[k]) : max(v[k], o[k]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < NPL; k++) {
+          const int kp = flip ? k ^ (size - 1) : k ^ j;
+          if (k < kp) {
+            const unsigned lo = min(v[k], v[kp]), hi = max(v[k], v[kp]);
+            v[k] = lo;
+            v[kp] = hi;
           }
         }
       }
@@ -369,10 +376,32 @@ __device__ __forceinline__ void warp_bitonic_sort_blocked(uint64_t (&v)[NPL], in
   }
 }
 
-__device__ __forceinline__ int64_t warp_sum_i64(int64_t x) {
+// Exact order of the rank records where truncated keys left neighbours
+// descending: odd-even transposition on |lambda| (equal values keep their
+// order, the lower bit first).  About 0.5% of 64-bit words need it, a pass or
+// two each.
+template <int NPL>
+__device__ __forceinline__ void fix_rank_order(RankBit *rb, int n, int lane) {
+  int moved;
+  do {
+    moved = 0;
+#pragma unroll 1
+    for (int ph = 0; ph < 2; ph++) {
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(FULL, x, d);
-  return x;
+      for (int x = 0; x < (NPL + 1) / 2; x++) {
+        const int p = 2 * (lane + 32 * x) + ph;
+        if (p + 1 < n) {
+          const RankBit u = rb[p], v = rb[p + 1];
+          if (u.a > v.a) {
+            rb[p] = v;
+            rb[p + 1] = u;
+            moved = 1;
+          }
+        }
+      }
+      __syncwarp();
+    }
+  } while (__any_sync(FULL, moved));
 }
 
 __device__ __forceinline__ float warp_min_f(float x) {
@@ -382,36 +411,33 @@ __device__ __forceinline__ float warp_min_f(float x) {
 }
 
 // floor(v * 256 + 1/2) for v >= 0, saturating at 2^20 - 1.  Exact in FP32:
-// v * 256 is a power-of-two scaling, and below the saturation point x + 1/2
-// needs no rounding (x < 2^20 has an ulp of at most 2^-4).
-__device__ __forceinline__ int64_t quant256(float v) {
-  const float x = v * 256.f;
-  if (!(x < 1048576.f)) return (1 << 20) - 1;
-  return (int64_t)min((int)floorf(x + 0.5f), (1 << 20) - 1);
-}
+// v * 256 is a power-of-two scaling, and below the saturation point the sum
+// with 1/2 needs no rounding (x < 2^20 has an ulp of at most 2^-4).
+__device__ __forceinline__ int quant256(float v) { return __float2int_rd(fminf(fmaf(v, 256.f, 0.5f), 1048575.5f)); }
 
 // 1-line ORBGRAND parameter: intercept/slope of the least-squares line through
 // (r, a_r), r = 1..n, rounded half up, clamped to [0, c_max]; 0 if the slope
-// is not positive.  All lanes get the same value.
-__device__ __forceinline__ int one_line_c(int64_t sy, int64_t sxy, int n, int c_max) {
-  int64_t sx = (int64_t)n * (n + 1) / 2;
-  int64_t sxx = (int64_t)n * (n + 1) * (2 * n + 1) / 6;
-  int64_t D = (int64_t)n * sxx - sx * sx;
-  int64_t Nb = (int64_t)n * sxy - sx * sy;
-  if (Nb <= 0) return 0;
-  int64_t num = sy * D - Nb * sx;
-  int64_t top = 2 * num + (int64_t)n * Nb;
-  if (top < 0) return 0;
-  // floor(top / den) clamped to c_max: an FP32 estimate (the hardware
-  // reciprocal: a few ulp) corrected with exact integer products (the
-  // quotient that matters is at most c_max <= 128)
-  const int64_t den = 2 * (int64_t)n * Nb;
-  if (top >= (int64_t)(c_max + 1) * den) return c_max;
-  int64_t c = (int64_t)__fdividef((float)top, (float)den);
-  c = c < 0 ? 0 : (c > c_max ? c_max : c);
-  while (c > 0 && c * den > top) c--;
-  while (c < c_max && (c + 1) * den <= top) c++;
-  return (int)c;
+// is not positive.  With sy = sum a_r, sxy = sum r a_r and B = 2 sxy -
+// (n + 1) sy (the slope is 6 B / (n (n^2 - 1))), intercept / slope + 1/2 =
+// (sy (n^2 - 1) - 3 n B) / (6 B) exactly, so the parameter is the number of
+// c = 1 .. c_max with 6 B c <= sy (n^2 - 1) - 3 n B: one candidate a lane,
+// counted by a ballot (the quotient by floating-point estimate and exact
+// correction was four times the instructions).  |sxy| < 2^34, so every
+// product fits 64 bits.  All lanes get the same value.
+template <int NPL>
+__device__ __forceinline__ int one_line_c(unsigned sy, int64_t sxy, int n, int c_max, int lane) {
+  const int64_t B = 2 * sxy - (int64_t)(n + 1) * sy;
+  if (B <= 0) return 0;
+  const int64_t den = 6 * B, top = (int64_t)sy * (n * n - 1) - 3 * n * B;
+  int c = 0;
+#pragma unroll 1
+  for (int k = 0; k < NPL; k++) {
+    const int cand = lane + 1 + 32 * k;
+    const unsigned ok = __ballot_sync(FULL, cand <= c_max && den * cand <= top);
+    c += __popc(ok);
+    if (ok != FULL) break;  // the candidates that pass are the smallest ones
+  }
+  return c;
 }
 
 // rank k (0-based position in the pattern) of a table entry: byte k + 1
@@ -458,11 +484,12 @@ __device__ __forceinline__ SYN ent_syndrome(const uint4 &e, int w, int wmax, con
   return s;
 }
 
-// sum over the pattern's ranks of a per-rank float
-__device__ __forceinline__ float ent_sum(const uint4 &e, int w, const float *x) {
+// sum over the pattern's ranks of |lambda| log2(e)
+template <int NPL, class SYN>
+__device__ __forceinline__ float ent_sum(const uint4 &e, int w, const Scratch<NPL, SYN> &sc) {
   float s = 0.f;
 #define SG_S(K) \
-  if (K < w) s += x[ent_rank<K>(e)];
+  if (K < w) s += sc.l2(ent_rank<K>(e));
   SG_S(0) SG_S(1) SG_S(2) SG_S(3) SG_S(4) SG_S(5) SG_S(6) SG_S(7)
   SG_S(8) SG_S(9) SG_S(10) SG_S(11) SG_S(12) SG_S(13) SG_S(14)
 #undef SG_S
@@ -472,132 +499,67 @@ __device__ __forceinline__ float ent_sum(const uint4 &e, int w, const float *x) 
 // ----------------------------------------------------------------------------
 // remaining mass: tail over cost > Cs (DP) + unqueried rest of level Cs
 // ----------------------------------------------------------------------------
-// Register form of the rank DP for Cs < 32 * SLOTS: lane l holds the head
-// masses of cost j = 32 s + l (s < SLOTS) for both parities; the shift by
-// d_e = e + 1 + c is a shuffle from lane (l - d) mod 32 plus a slot select.
-template <class Ops, int SLOTS>
-__device__ __forceinline__ void dp_regs(int Cs, int c, int R0, int cls, const typename Ops::T *sfac,
-                                        const typename Ops::T *fu, const typename Ops::T *fb, const float *ek,
-                                        typename Ops::T g_even, typename Ops::T g_odd, int lane,
-                                        typename Ops::T &acc) {
-  using T = typename Ops::T;
-  constexpr bool SCALED = sizeof(T) == 4;
-  T he[SLOTS], ho[SLOTS];
-#pragma unroll
-  for (int t = 0; t < SLOTS; t++) {
-    he[t] = (t == 0 && lane == 0) ? Ops::one() : Ops::zero();
-    ho[t] = Ops::zero();
-  }
-  for (int e = 0; e < R0; e++) {
-    const int d = e + 1 + c;
-    const T s = sfac[e];
-    const T Fb = fb[e + 1];
-    const T F1u = Ops::add(Ops::one(), fu[e + 1]);
-    const int dq = d >> 5, dr = d & 31;
-    const int src = (lane - dr) & 31;
-    const int back = dq + (lane < dr ? 1 : 0);  // source slot = sl - back
-    T she[SLOTS], sho[SLOTS];
-#pragma unroll
-    for (int t = 0; t < SLOTS; t++) {
-      she[t] = Ops::shfl(he[t], src);
-      sho[t] = Ops::shfl(ho[t], src);
-    }
-#pragma unroll
-    for (int sl = 0; sl < SLOTS; sl++) {
-      const int j = sl * 32 + lane;
-      if (j <= Cs) {
-        if (j > Cs - d) {
-          T w = s;
-          if constexpr (SCALED) w = Ops::mul(w, Ops::from_float(ek[j + d - Cs]));
-          T term;
-          if (cls == 0)
-            term = Ops::add(Ops::mul(he[sl], Fb), Ops::mul(ho[sl], F1u));
-          else if (cls == 1)
-            term = Ops::add(Ops::mul(he[sl], F1u), Ops::mul(ho[sl], Fb));
-          else
-            term = Ops::mul(Ops::add(he[sl], ho[sl]), Ops::add(F1u, Fb));
-          acc = Ops::fma(w, term, acc);
-        }
-        if (j >= d) {
-          const int ss = sl - back;
-          T pe = Ops::zero(), po = Ops::zero();
-#pragma unroll
-          for (int t = 0; t < SLOTS; t++)
-            if (t == ss) {
-              pe = she[t];
-              po = sho[t];
-            }
-          he[sl] = Ops::fma(s, po, he[sl]);
-          ho[sl] = Ops::fma(s, pe, ho[sl]);
-        }
-      }
-    }
-#ifdef SG_PHASE_PROFILE
-    if (lane == 0) SG_PROF(7, 1);
-#endif
-  }
-  // high ranks (d_e > Cs) joined to every head pattern
-#pragma unroll
-  for (int sl = 0; sl < SLOTS; sl++) {
-    const int j = sl * 32 + lane;
-    if (j <= Cs) {
-      T w = Ops::one();
-      if constexpr (SCALED) w = Ops::from_float(ek[j]);
-      T term;
-      if (cls == 0)
-        term = Ops::add(Ops::mul(he[sl], g_even), Ops::mul(ho[sl], g_odd));
-      else if (cls == 1)
-        term = Ops::add(Ops::mul(he[sl], g_odd), Ops::mul(ho[sl], g_even));
-      else
-        term = Ops::mul(Ops::add(he[sl], ho[sl]), Ops::add(g_even, g_odd));
-      acc = Ops::fma(w, term, acc);
-    }
-  }
-}
-
-// Shared-memory form of the same DP for large stop levels (out of line: rare).
+// The rank DP: he/ho hold the head masses of cost j = 0..Cs by parity, in the
+// block's remaining-mass area; rank e lifts cost j by d_e = e + 1 + c.  Slots
+// of 32 costs, one cost a lane.  Every term is accumulated before the rank's
+// update, by ascending slots below a stop level of 128 (FP32) and by
+// descending ones otherwise.  Rolled and short: it runs for fewer than 1% of
+// the words, inside the words' kernels.
 template <class Ops>
-__device__ __noinline__ void dp_smem(int Cs, int c, int R0, int cls, const typename Ops::T *sfac, const typename Ops::T *fu,
-                        const typename Ops::T *fb, const float *ek, typename Ops::T g_even, typename Ops::T g_odd,
-                        typename Ops::T *he, typename Ops::T *ho, int lane, typename Ops::T &acc) {
+__device__ __forceinline__ void dp_ranks(int Cs, int c, int R0, int cls, const typename Ops::T *sfac,
+                                         const typename Ops::T *fu, const typename Ops::T *fb, const float *ek,
+                                         typename Ops::T g_even, typename Ops::T g_odd, typename Ops::T *he,
+                                         typename Ops::T *ho, int lane, typename Ops::T &acc) {
   using T = typename Ops::T;
   constexpr bool SCALED = sizeof(T) == 4;
+#pragma unroll 1
   for (int j = lane; j <= Cs; j += 32) {
     he[j] = j == 0 ? Ops::one() : Ops::zero();
     ho[j] = Ops::zero();
   }
   __syncwarp();
   const int nslot = (Cs + 32) >> 5;
-  for (int e = 0; e < R0; e++) {
+  const bool ascending = SCALED && Cs < 128;
+#pragma unroll 1
+  for (int e = 0; e <= R0; e++) {
+    // e < R0: rank e joins the heads; e == R0: the high ranks (d_e > Cs) join every head
+    const bool high = e == R0;
     const int d = e + 1 + c;
-    const T s = sfac[e];
-    const T Fb = fb[e + 1];
-    const T F1u = Ops::add(Ops::one(), fu[e + 1]);
+    const T s = high ? Ops::one() : sfac[e];
+    const T fe = high ? g_even : fb[e + 1];
+    const T fo = high ? g_odd : Ops::add(Ops::one(), fu[e + 1]);
+#pragma unroll 1
+    for (int t = 0; t < nslot; t++) {
+      const int j = 32 * (ascending || high ? t : nslot - 1 - t) + lane;
+      if (j <= Cs && (high || j > Cs - d)) {
+        T w = s;
+        if constexpr (SCALED) {
+          const T k = Ops::from_float(ek[high ? j : j + d - Cs]);
+          w = high ? k : Ops::mul(w, k);
+        }
+        const T a = he[j], b = ho[j];
+        T term;
+        if (cls == 0)
+          term = Ops::add(Ops::mul(a, fe), Ops::mul(b, fo));
+        else if (cls == 1)
+          term = Ops::add(Ops::mul(a, fo), Ops::mul(b, fe));
+        else
+          term = Ops::mul(Ops::add(a, b), Ops::add(fo, fe));
+        acc = Ops::fma(w, term, acc);
+      }
+    }
+    __syncwarp();
+    if (high) break;
     // slots from the top, so every read of he/ho[j - d] sees the values
     // before this rank (a slot's reads are separated from its writes)
+#pragma unroll 1
     for (int sl = nslot - 1; sl >= 0; sl--) {
       const int j = sl * 32 + lane;
+      const bool upd = j <= Cs && j >= d;
       T ne = Ops::zero(), no = Ops::zero();
-      const bool inr = j <= Cs;
-      const bool upd = inr && j >= d;
-      if (inr) {
-        const T hej = he[j], hoj = ho[j];
-        if (j > Cs - d) {
-          T w = s;
-          if constexpr (SCALED) w = Ops::mul(w, Ops::from_float(ek[j + d - Cs]));
-          T term;
-          if (cls == 0)
-            term = Ops::add(Ops::mul(hej, Fb), Ops::mul(hoj, F1u));
-          else if (cls == 1)
-            term = Ops::add(Ops::mul(hej, F1u), Ops::mul(hoj, Fb));
-          else
-            term = Ops::mul(Ops::add(hej, hoj), Ops::add(F1u, Fb));
-          acc = Ops::fma(w, term, acc);
-        }
-        if (upd) {
-          ne = Ops::fma(s, ho[j - d], hej);
-          no = Ops::fma(s, he[j - d], hoj);
-        }
+      if (upd) {
+        ne = Ops::fma(s, ho[j - d], he[j]);
+        no = Ops::fma(s, he[j - d], ho[j]);
       }
       __syncwarp();
       if (upd) {
@@ -606,28 +568,19 @@ __device__ __noinline__ void dp_smem(int Cs, int c, int R0, int cls, const typen
       }
       __syncwarp();
     }
+#ifdef SG_PHASE_PROFILE
+    if (lane == 0) SG_PROF(7, 1);
+#endif
   }
-  for (int j = lane; j <= Cs; j += 32) {
-    T w = Ops::one();
-    if constexpr (SCALED) w = Ops::from_float(ek[j]);
-    T term;
-    if (cls == 0)
-      term = Ops::add(Ops::mul(he[j], g_even), Ops::mul(ho[j], g_odd));
-    else if (cls == 1)
-      term = Ops::add(Ops::mul(he[j], g_odd), Ops::mul(ho[j], g_even));
-    else
-      term = Ops::mul(Ops::add(he[j], ho[j]), Ops::add(g_even, g_odd));
-    acc = Ops::fma(w, term, acc);
-  }
-  __syncwarp();
 }
 
 // The (scaled) remaining mass summed over the warp.  With FOps every mass
 // carries the factor 2^(g2 * Cs) (g2 = gamma log2 e); with XOps g2 = 0.
-// `qs` is the order-table index of the last queried pattern.
+// `ent` and `cost` are the word's order, `tc` its entries, `qs` the last queried pattern.
 template <class Ops, int NPL, class SYN>
-__device__ __noinline__ typename Ops::T remaining_scaled(const Scratch<NPL, SYN> &sc, const DevOrder &O, int tb, int tc, int qs,
-                                            int n, int c, int cls, int Cs, float g2, int lane) {
+__device__ __forceinline__ typename Ops::T remaining_scaled(const Scratch<NPL, SYN> &sc, const uint4 *ent,
+                                                            const uint16_t *cost, int tc, int qs, int n, int c,
+                                                            int cls, int Cs, float g2, int lane) {
   using T = typename Ops::T;
   constexpr int NT = 32 * NPL;
   T *sfac = reinterpret_cast<T *>(sc.tail());
@@ -645,10 +598,10 @@ __device__ __noinline__ typename Ops::T remaining_scaled(const Scratch<NPL, SYN>
   for (int q0 = qs + 1; q0 < tc; q0 += 32) {
     const int q = q0 + lane;
     bool in = false;
-    if (q < tc) in = __ldg(O.cost + tb + q) == (uint16_t)Cs;
+    if (q < tc) in = __ldg(cost + q) == (uint16_t)Cs;
     if (in) {
-      const uint4 e = __ldg(O.ent + tb + q);
-      const float s2 = ent_sum(e, e.x & 0xff, sc.l2());
+      const uint4 e = __ldg(ent + q);
+      const float s2 = ent_sum<NPL, SYN>(e, e.x & 0xff, sc);
       acc = Ops::add(acc, Ops::from_log2(g2Cs - s2));
     }
     if (!__all_sync(FULL, in)) break;  // costs are nondecreasing
@@ -665,10 +618,10 @@ __device__ __noinline__ typename Ops::T remaining_scaled(const Scratch<NPL, SYN>
       const int e = lane * NPL + k;
       T t = Ops::zero();
       if (e < n) {
-        t = Ops::from_log2(-sc.l2()[e]);
+        t = Ops::from_log2(-sc.l2(e));
         // factor used by the tail: low ranks t * 2^(g2 d_e), high ranks t * 2^(g2 Cs)
         const float d = (float)(e + 1 + c);
-        sfac[e] = Ops::from_log2((e < R0 ? g2 * d : g2Cs) - sc.l2()[e]);
+        sfac[e] = Ops::from_log2((e < R0 ? g2 * d : g2Cs) - sc.l2(e));
       }
       const T nu = Ops::fma(b, t, u);
       const T nb = Ops::fma(u, t, Ops::add(b, t));
@@ -725,46 +678,26 @@ __device__ __noinline__ typename Ops::T remaining_scaled(const Scratch<NPL, SYN>
   }
 
   // --- low ranks in ascending order: tail contributions and the cost DP
-  bool done = false;
-  if constexpr (SCALED) {
-    if (Cs < 64) {
-      dp_regs<Ops, 2>(Cs, c, R0, cls, sfac, fu, fb, ek, g_even, g_odd, lane, acc);
-      done = true;
-    } else if (Cs < 128) {
-      dp_regs<Ops, 4>(Cs, c, R0, cls, sfac, fu, fb, ek, g_even, g_odd, lane, acc);
-      done = true;
-    }
-  }
-  if (!done) {
-#ifdef SG_PHASE_PROFILE
-    if (lane == 0) SG_PROF(9, 1);
-#endif
-    dp_smem<Ops>(Cs, c, R0, cls, sfac, fu, fb, ek, g_even, g_odd, he, ho, lane, acc);
-  }
+  dp_ranks<Ops>(Cs, c, R0, cls, sfac, fu, fb, ek, g_even, g_odd, he, ho, lane, acc);
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) acc = Ops::add(acc, Ops::shfl_xor(acc, d));
   __syncwarp();
   return acc;
 }
 
-// Extended-range evaluation (out of line: only when every FP32-scaled term
-// of the dominant part underflows).
-template <int NPL, class SYN>
-__device__ __noinline__ float remaining_log2_xf(const Scratch<NPL, SYN> &sc, const DevOrder &O, int tb, int tc, int qs,
-                                                int n, int c, int cls, int Cs, int lane) {
-  const XF x = remaining_scaled<XOps, NPL, SYN>(sc, O, tb, tc, qs, n, c, cls, Cs, 0.f, lane);
-  return __shfl_sync(FULL, xf_log2(x), 0);
-}
-
 // Class total of the nonzero patterns in double-float: prod_e (1 + y t_e) as
-// (even part - 1, odd part), lanes own ranks lane*NPL .. lane*NPL+NPL-1, then
-// a butterfly over the warp; lane 0's result is broadcast.  Every term is
-// nonnegative, so the additions need no cancellation handling.
+// (even part - 1, odd part) = (u, b), lanes own ranks lane*NPL ..
+// lane*NPL+NPL-1, then a tree over the warp whose root (lane 0's chain) is
+// broadcast.  Every term is nonnegative, so the additions need no
+// cancellation handling.  Joining two nodes takes the same operations for u
+// as for b on other operands, and a level of the tree needs at most 16
+// joins: lanes 0-15 form the u parts and lanes 16-31 the b parts, so a level
+// is 47 double-float instructions instead of 94, executed and fetched.
 template <int NPL, class SYN>
-__device__ __noinline__ DF class_total_df(const Scratch<NPL, SYN> &sc, int n, int cls, int lane) {
-  DF u = {0.f, 0.f}, b = {0.f, 0.f};
-#pragma unroll
-  for (int k = 0; k < NPL; k++) {
+__device__ __forceinline__ DF class_total_df(const Scratch<NPL, SYN> &sc, int n, int cls, int lane) {
+  DF u = {0.f, 0.f}, b = {lane * NPL < n ? sc.hr()[lane * NPL].t : 0.f, 0.f};
+#pragma unroll 1
+  for (int k = 1; k < NPL; k++) {
     const int e = lane * NPL + k;
     if (e < n) {
       const float t = sc.hr()[e].t;
@@ -774,110 +707,145 @@ __device__ __noinline__ DF class_total_df(const Scratch<NPL, SYN> &sc, int n, in
       b = nb;
     }
   }
+  const bool odd = lane >= 16;
+  DF v = odd ? b : u, w = odd ? u : b;  // own part, other part of the own node
+  DF vo, wo;                            // the same parts of the node to join
 #pragma unroll 1
   for (int d = 16; d > 0; d >>= 1) {
-    const DF ou = {__shfl_xor_sync(FULL, u.h, d), __shfl_xor_sync(FULL, u.l, d)};
-    const DF ob = {__shfl_xor_sync(FULL, b.h, d), __shfl_xor_sync(FULL, b.l, d)};
-    const DF nu = df_add_pos(df_add_pos(u, ou), df_add_pos(df_mul(u, ou), df_mul(b, ob)));
-    const DF nb = df_add_pos(df_add_pos(b, ob), df_add_pos(df_mul(u, ob), df_mul(b, ou)));
-    u = nu;
-    b = nb;
+    if (d == 16) {  // every lane still holds both parts of its own node
+      const DF xu = {__shfl_xor_sync(FULL, u.h, 16), __shfl_xor_sync(FULL, u.l, 16)};
+      const DF xb = {__shfl_xor_sync(FULL, b.h, 16), __shfl_xor_sync(FULL, b.l, 16)};
+      if (odd) {  // this lane's node is the upper one of the pair (lane - 16, lane)
+        vo = b;
+        wo = u;
+        v = xb;
+        w = xu;
+      } else {
+        vo = xu;
+        wo = xb;
+      }
+    } else {
+      w = DF{__shfl_xor_sync(FULL, v.h, 16), __shfl_xor_sync(FULL, v.l, 16)};
+      vo = DF{__shfl_xor_sync(FULL, v.h, d), __shfl_xor_sync(FULL, v.l, d)};
+      wo = DF{__shfl_xor_sync(FULL, w.h, d), __shfl_xor_sync(FULL, w.l, d)};
+    }
+    // u: (u + ou) + (u ou + b ob);  b: (b + ob) + (u ob + b ou)
+    const DF pu = odd ? w : v, pb = odd ? v : w;
+    v = df_add_pos(df_add_pos(v, vo), df_add_pos(df_mul(pu, vo), df_mul(pb, wo)));
   }
-  const DF E = cls == 0 ? u : (cls == 1 ? b : df_add_pos(u, b));
-  return {__shfl_sync(FULL, E.h, 0), __shfl_sync(FULL, E.l, 0)};
+  u = DF{__shfl_sync(FULL, v.h, 0), __shfl_sync(FULL, v.l, 0)};
+  b = DF{__shfl_sync(FULL, v.h, 16), __shfl_sync(FULL, v.l, 16)};
+  return cls == 0 ? u : (cls == 1 ? b : df_add_pos(u, b));
 }
 
 // The unqueried patterns summed directly: the cost DP of remaining_scaled
-// under the block's lock.  Out of line: the DP runs for 0.04-0.9% of the
-// component words, and as a call it keeps the two call sites of
-// remaining_log2 short (1-1.5% faster than inline for eBCH(32,26), (64,51)
-// and (128,120) at 7 blocks per SM; within 1% for eBCH(64,57)).
+// under the block's lock, again in the extended range when every FP32-scaled
+// term of the dominant part underflows.  It runs for 0.04-0.9% of the
+// component words; inlined all the same, because an out-of-line call keeps
+// the whole word's values in the registers that calls preserve (63 spill
+// loads a word at 40 registers) and leaves the compiler unsure that the warp
+// comes back converged.
+// Returns log2 of the mass and flags: bit 0 when the extended-range sum was
+// needed, bit 1 when the block's remaining-mass area could not be locked.
+struct Remaining {
+  float lr2;
+  int flags;
+};
 template <int NPL, class SYN>
-__device__ __noinline__ float remaining_log2_dp(const Scratch<NPL, SYN> &sc, const DevOrder &O, int tb, int tc,
-                                                int qs, int n, int c, int cls, int lane, int *used_xf) {
+__device__ __forceinline__ Remaining remaining_log2_dp(const Scratch<NPL, SYN> &sc, const uint4 *ent,
+                                                       const uint16_t *cost, int tc, int qs, int n, int c, int cls,
+                                                       int lane) {
 #ifdef SG_PHASE_PROFILE
   if (lane == 0) SG_PROF(6, 1);
 #endif
-  const int Cs = __ldg(O.cost + tb + qs);
+  const int Cs = __ldg(cost + qs);
   const int R0 = min(max(Cs - c, 0), n);
   float g = CUDART_INF_F;
-  for (int e = lane; e < R0; e += 32) g = fminf(g, sc.l2()[e] / (float)(e + 1 + c));
+  for (int e = lane; e < R0; e += 32) g = fminf(g, sc.l2(e) / (float)(e + 1 + c));
   g = __shfl_sync(FULL, warp_min_f(g), 0);
   if (!(g < CUDART_INF_F)) g = 0.f;
   const bool held = dp_lock(sc.lock(), lane);
-  float out;
-  const float tot = __shfl_sync(FULL, remaining_scaled<FOps, NPL, SYN>(sc, O, tb, tc, qs, n, c, cls, Cs, g, lane), 0);
+  Remaining out = {0.f, 0};
+  const float tot =
+      __shfl_sync(FULL, remaining_scaled<FOps, NPL, SYN>(sc, ent, cost, tc, qs, n, c, cls, Cs, g, lane), 0);
   if (tot >= 0x1p-60f && tot < CUDART_INF_F) {
-    out = log2f(tot) - g * (float)Cs;
+    out.lr2 = log2f(tot) - g * (float)Cs;
   } else {
-    if (used_xf) *used_xf |= 1;
+    out.flags = 1;
 #ifdef SG_PHASE_PROFILE
     if (lane == 0) SG_PROF(8, 1);
 #endif
-    out = remaining_log2_xf<NPL, SYN>(sc, O, tb, tc, qs, n, c, cls, Cs, lane);
+    out.lr2 = __shfl_sync(
+        FULL, xf_log2(remaining_scaled<XOps, NPL, SYN>(sc, ent, cost, tc, qs, n, c, cls, Cs, 0.f, lane)), 0);
   }
   dp_unlock(sc.lock(), held, lane);
-  if (!held && used_xf) *used_xf |= 2;
+  if (!held) out.flags |= 2;
   return out;
 }
 
 // log2 of the remaining (unqueried) mass relative to p(0^n|r); warp-uniform.
-// *used_xf (if given) gets bit 0 when the extended-range sum was needed and
-// bit 1 when the block's remaining-mass area could not be locked.
 // tq is the queried mass of the nonzero patterns (double-float, summed over
 // the warp, the same value in every lane).  The class total minus tq is used
 // when it is well conditioned: in FP32 when the difference is at least 2% of
 // the operands (FP32 rounding of about 4e-6 of them moves it by at most 2e-4
 // relative), in double-float when it is at least 2^-26 of them (rounding of a
 // few 2^-46 moves it by at most about 1e-5 relative).  Otherwise the
-// unqueried patterns are summed directly.
-template <int NPL, class SYN>
-__device__ float remaining_log2(const Scratch<NPL, SYN> &sc, const DevOrder &O, int tb, int tc, int qs, int n, int c,
-                                int cls, int lane, DF tq, int *used_xf) {
+// unqueried patterns are summed directly.  KEEP: the double-float class total
+// is kept with the word's head (the threshold rule asks at every listed word).
+template <bool KEEP, int NPL, class SYN>
+__device__ __forceinline__ Remaining remaining_log2(const Scratch<NPL, SYN> &sc, const uint4 *ent,
+                                                    const uint16_t *cost, int tc, int qs, int n, int cls, int lane,
+                                                    DF tq) {
   // class total of the nonzero patterns: prod_e (1 + y t_e) as (even - 1, odd)
-  {
-    float u = 0.f, b = 0.f;
+  float u = 0.f, b = 0.f;
 #pragma unroll
-    for (int k = 0; k < NPL; k++) {
-      const int e = lane * NPL + k;
-      if (e < n) {
-        const float t = sc.hr()[e].t;
-        const float nu = fmaf(b, t, u), nb = fmaf(u, t, b + t);
-        u = nu;
-        b = nb;
-      }
-    }
-#pragma unroll 1
-    for (int d = 16; d > 0; d >>= 1) {
-      const float ou = __shfl_xor_sync(FULL, u, d), ob = __shfl_xor_sync(FULL, b, d);
-      const float nu = (u + ou) + fmaf(u, ou, b * ob);
-      const float nb = (b + ob) + fmaf(u, ob, b * ou);
+  for (int k = 0; k < NPL; k++) {
+    const int e = lane * NPL + k;
+    if (e < n) {
+      const float t = sc.hr()[e].t;
+      const float nu = fmaf(b, t, u), nb = fmaf(u, t, b + t);
       u = nu;
       b = nb;
     }
-    // the butterfly's fused products round differently per lane: take lane
-    // 0's value so the branch below is warp-uniform
-    u = __shfl_sync(FULL, u, 0);
-    b = __shfl_sync(FULL, b, 0);
-    const float enz = cls == 0 ? u : (cls == 1 ? b : u + b);
-    const float tqf = tq.h + tq.l;
-    const float r = enz - tqf;
-    const bool in_range = enz > 0x1p-60f && enz < 0x1p60f;
-    // the hardware log2 (about 2^-22 relative): far inside the soft output's tolerance
-    if (in_range && r > 0.02f * (enz + tqf)) return __log2f(r);
-    if (in_range) {
-      const DF E = class_total_df<NPL, SYN>(sc, n, cls, lane);
-      const DF R = df_add(E, DF{-tq.h, -tq.l});
-#ifdef SG_PHASE_PROFILE
-      if (lane == 0) SG_PROF(R.h > 0x1p-26f * (E.h + tq.h) ? 12 : 13, 1);
-#endif
-      if (R.h > 0x1p-26f * (E.h + tq.h)) return __log2f(R.h + R.l);
-    }
-#ifdef SG_PHASE_PROFILE
-    if (!in_range && lane == 0) SG_PROF(15, 1);
-#endif
   }
-  return remaining_log2_dp<NPL, SYN>(sc, O, tb, tc, qs, n, c, cls, lane, used_xf);
+#pragma unroll 1
+  for (int d = 16; d > 0; d >>= 1) {
+    const float ou = __shfl_xor_sync(FULL, u, d), ob = __shfl_xor_sync(FULL, b, d);
+    const float nu = (u + ou) + fmaf(u, ou, b * ob);
+    const float nb = (b + ob) + fmaf(u, ob, b * ou);
+    u = nu;
+    b = nb;
+  }
+  // the butterfly's fused products round differently per lane: take lane
+  // 0's value so the branches below are warp-uniform
+  const float enz = __shfl_sync(FULL, cls == 0 ? u : (cls == 1 ? b : u + b), 0);
+  const float tqf = tq.h + tq.l;
+  const float r = enz - tqf;
+  if (enz > 0x1p-60f && enz < 0x1p60f) {
+    // the hardware log2 (about 2^-22 relative): far inside the soft output's tolerance
+    if (r > 0.02f * (enz + tqf)) return {__log2f(r), 0};
+    DF E;
+    unsigned *kept = sc.headv() + NPL + 1;
+    if (KEEP && sc.head_at(NPL + 1)) {
+      E = DF{__uint_as_float(sc.head_at(NPL + 2)), __uint_as_float(sc.head_at(NPL + 3))};
+    } else {
+      E = class_total_df<NPL, SYN>(sc, n, cls, lane);
+      if (KEEP) {
+        if (lane == 0) {
+          kept[0] = 1u;
+          kept[1] = __float_as_uint(E.h);
+          kept[2] = __float_as_uint(E.l);
+        }
+        __syncwarp();
+      }
+    }
+    const DF R = df_add(E, DF{-tq.h, -tq.l});
+#ifdef SG_PHASE_PROFILE
+    if (lane == 0) SG_PROF(R.h > 0x1p-26f * (E.h + tq.h) ? 12 : 13, 1);
+#endif
+    if (R.h > 0x1p-26f * (E.h + tq.h)) return {__log2f(R.h + R.l), 0};
+  }
+  return remaining_log2_dp<NPL, SYN>(sc, ent, cost, tc, qs, n, (int)sc.head_at(NPL), cls, lane);
 }
 
 // numerically safe log(exp(a) + exp(b)) (natural log, -inf aware)
@@ -899,30 +867,32 @@ struct WordHead {
   int c;             // 1-line parameter
 };
 
-// Hard decision, parity, syndrome of y, reliability ranks (scratch al/l2/
-// perm/hs) and the 1-line parameter.  Returns false (and leaves the head
-// undefined) if any input is not finite.
+// Hard decision, parity, syndrome of y, reliability ranks (scratch rb/hr) and
+// the 1-line parameter.  The caller has stored lambda in sc.lamv().  Returns
+// false (and leaves the head undefined) if any input is not finite.
 template <int NPL, class SYN>
-__device__ bool siso_prologue(const DevCode &code, const Scratch<NPL, SYN> &sc, const float (&lam)[NPL], int lane,
-                              WordHead<NPL, SYN> &h) {
+__device__ __forceinline__ bool siso_prologue(const DevCode &code, const Scratch<NPL, SYN> &sc, const float (&lam)[NPL],
+                                              int lane, WordHead<NPL, SYN> &h) {
   const int n = code.n;
+  const SYN *hcol = reinterpret_cast<const SYN *>(code.hcol);  // 8-byte columns: the low half serves 32-bit syndromes
+  constexpr int HS = 8 / sizeof(SYN);
   bool bad = false;
 #pragma unroll
   for (int k = 0; k < NPL; k++)
-    if (lane + 32 * k < n && !isfinite(lam[k])) bad = true;
+    if (lane + 32 * k < n && !(fabsf(lam[k]) < CUDART_INF_F)) bad = true;
   if (__any_sync(FULL, bad)) return false;
 
-  int par = 0;
+  int ones = 0;
   SYN s0p = 0;
 #pragma unroll
   for (int k = 0; k < NPL; k++) {
     const int i = lane + 32 * k;
     const bool one = (i < n) && lam[k] < 0.f;  // lambda = 0 -> bit 0
     h.yb[k] = __ballot_sync(FULL, one);
-    par ^= __popc(h.yb[k]) & 1;
-    if (one) s0p ^= (SYN)__ldg(code.hcol + i);
+    ones += __popc(h.yb[k]);
+    if (one) s0p ^= __ldg(hcol + i * HS);
   }
-  h.par = par;
+  h.par = ones & 1;
   if (sizeof(SYN) == 4) {
     h.s0 = (SYN)__reduce_xor_sync(FULL, (unsigned)s0p);
   } else {
@@ -931,36 +901,50 @@ __device__ bool siso_prologue(const DevCode &code, const Scratch<NPL, SYN> &sc, 
     h.s0 = (SYN)(((uint64_t)hi_ << 32) | lo_);
   }
 
-  // reliability ranks: sort (|lambda|, index) ascending
-  uint64_t key[NPL];
+  // reliability ranks: sort (|lambda|, index) ascending, on 32-bit keys of
+  // |lambda| (its lowest LOGN - 1 mantissa bits dropped) and the index; equal
+  // values are in index order, and neighbours that the dropped bits would
+  // order otherwise are found by comparing the exact values and exchanged
+  constexpr int LOGN = NPL == 1 ? 5 : (NPL == 2 ? 6 : 7);
+  unsigned key[NPL];
 #pragma unroll
   for (int k = 0; k < NPL; k++) {
     const int i = lane + 32 * k;
-    key[k] = i < n ? (((uint64_t)__float_as_uint(fabsf(lam[k])) << 32) | (uint64_t)i) : ~0ull;
+    key[k] = i < n ? (((__float_as_uint(lam[k]) << 1) >> LOGN) << LOGN) | i : 0xffffffffu;
   }
-  warp_bitonic_sort_blocked<NPL>(key, lane);
-  int64_t sy = 0, sxy = 0;
+  warp_sort_blocked<NPL>(key, lane);
+  __syncwarp();  // lambda is in shared memory (siso_word)
+  float a[NPL];
+  bool wrong = false;
+#pragma unroll
+  for (int k = 0; k < NPL; k++) {
+    const int bit = key[k] & (32 * NPL - 1);
+    a[k] = fabsf(sc.lamv()[bit]);
+    sc.rb()[lane * NPL + k] = RankBit{a[k], bit};
+    if (k > 0 && lane * NPL + k < n) wrong = wrong || a[k - 1] > a[k];
+  }
+  const float next = __shfl_down_sync(FULL, a[0], 1);
+  if (lane < 31 && lane * NPL + NPL < n) wrong = wrong || a[NPL - 1] > next;
+  if (__any_sync(FULL, wrong)) {
+    __syncwarp();
+    fix_rank_order<NPL>(sc.rb(), n, lane);
+  }
+  unsigned sy = 0, sxy = 0;  // a lane's share: below 2^22 and 2^29
 #pragma unroll
   for (int k = 0; k < NPL; k++) {
     const int e = lane * NPL + k;  // sorted position (blocked layout)
     if (e < n) {
-      const float a = __uint_as_float((unsigned)(key[k] >> 32));
-      const int idx = (int)(key[k] & 0xffffffffu);
-      const float l2v = __fmul_rn(a, LOG2E_F);
-      sc.al()[e] = a;
-      sc.l2()[e] = l2v;
-      sc.perm()[e] = (uint8_t)idx;
-      sc.hr()[e] = RankRec<SYN>{(SYN)__ldg(code.hcol + idx), exp2f(-l2v)};
-      const int64_t qa = quant256(a);
+      const RankBit r = sc.rb()[e];
+      sc.hr()[e] = RankRec<SYN>{__ldg(hcol + r.bit * HS), exp2f(-__fmul_rn(r.a, LOG2E_F))};
+      const unsigned qa = (unsigned)quant256(r.a);
       sy += qa;
       sxy += qa * (e + 1);
     }
   }
-  // sy < 2^27 fits one 32-bit reduction; sxy < 2^34 is split at bit 24
-  sy = (int64_t)__reduce_add_sync(FULL, (unsigned)sy);
-  sxy = ((int64_t)__reduce_add_sync(FULL, (unsigned)(sxy >> 24)) << 24) +
-        (int64_t)__reduce_add_sync(FULL, (unsigned)(sxy & 0xffffff));
-  h.c = one_line_c(sy, sxy, n, code.c_max);
+  // the sum of sy is below 2^27; that of sxy (below 2^34) is taken in two parts
+  sy = __reduce_add_sync(FULL, sy);
+  const int64_t sxyw = ((int64_t)__reduce_add_sync(FULL, sxy >> 16) << 16) + __reduce_add_sync(FULL, sxy & 0xffffu);
+  h.c = one_line_c<NPL>(sy, sxyw, n, code.c_max, lane);
   if (lane == 0) sc.hr()[n] = RankRec<SYN>{(SYN)0, 1.f};  // neutral record for unused entry bytes
   __syncwarp();
   return true;
@@ -1085,6 +1069,8 @@ __device__ int trace_word(const DevCode &code, const Scratch<NPL, SYN> &sc, cons
                           int max_q, uint64_t *out, int *c_out) {
   constexpr int NM = (32 * NPL + 63) / 64;
   WordHead<NPL, SYN> h;
+#pragma unroll
+  for (int k = 0; k < NPL; k++) sc.lamv()[lane + 32 * k] = lam[k];
   if (!siso_prologue<NPL, SYN>(code, sc, lam, lane, h)) return -1;
   const DevOrder &O = code.ord;
   const int ti = h.c * O.ncls + (code.even ? h.par : 0);
@@ -1115,52 +1101,12 @@ __device__ int trace_word(const DevCode &code, const Scratch<NPL, SYN> &sc, cons
   return qn;
 }
 
-__device__ __forceinline__ float warp_sum_f(float x) {
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(FULL, x, d);
-  return x;
-}
-
-// Record the hit of lane hl as list entry `slot`: the codeword y + z in bit
-// order (sc.cw()) and log p(z)/p(0) = -sum |lambda| over z (sc.lp()).  The
-// pattern is broadcast and lane k handles its k-th rank.
-template <int NPL, class SYN>
-__device__ __forceinline__ void record_hit(const Scratch<NPL, SYN> &sc, const WordHead<NPL, SYN> &h, const uint4 &e,
-                                           int hl, int slot, int lane) {
-  constexpr int NM = (32 * NPL + 63) / 64;
-  uint4 b;
-  b.x = __shfl_sync(FULL, e.x, hl);
-  b.y = __shfl_sync(FULL, e.y, hl);
-  b.z = __shfl_sync(FULL, e.z, hl);
-  b.w = __shfl_sync(FULL, e.w, hl);
-  const int w = b.x & 0xff;
-  const int byte = lane + 1;  // rank k = lane sits in byte k + 1
-  const unsigned wd = byte < 4 ? b.x : (byte < 8 ? b.y : (byte < 12 ? b.z : b.w));
-  const bool mine = lane < w;
-  const int r = mine ? (wd >> (8 * (byte & 3))) & 0xff : 0;
-  const float ls = warp_sum_f(mine ? sc.al()[r] : 0.f);
-  const int bi = mine ? sc.perm()[r] : 0;
-#pragma unroll
-  for (int k = 0; k < NPL; k++) {
-    const unsigned word = __reduce_or_sync(FULL, (mine && (bi >> 5) == k) ? 1u << (bi & 31) : 0u) ^ sc.head_at(k);
-    if (lane == 0) reinterpret_cast<unsigned *>(sc.cw() + slot * NM)[k] = word;
-  }
-  if (lane == 0) {
-    if (NPL & 1) reinterpret_cast<unsigned *>(sc.cw() + slot * NM)[NPL] = 0u;  // upper half of the last u64
-    sc.lp()[slot] = -ls;
-  }
-  __syncwarp();
-}
-
 // threshold rule: predicted probability that the list misses the codeword
 __device__ __forceinline__ bool thr_reached(const float *lp, int nhit, float M, float thr) {
   float D = M;
+#pragma unroll 1
   for (int l = 0; l < nhit; l++) D = lse(D, lp[l]);
   return expf(M - D) < thr;
-}
-template <int NPL, class SYN>
-__device__ __forceinline__ bool thr_reached(const Scratch<NPL, SYN> &sc, int nhit, float M, float thr) {
-  return thr_reached(sc.lp(), nhit, M, thr);
 }
 
 // eq. LLRi in the log domain for a bit whose linear sums underflowed (out of line: rare)
@@ -1178,155 +1124,130 @@ __device__ __noinline__ float lapp_logdomain(const Scratch<NPL, SYN> &sc, int nh
   return b0 - b1;
 }
 
-// The query loop when no threshold rule applies (thr = 0), out of line: its
-// register allocation is its own, not shaped by the rest of the word (inline,
-// the loop shared the word's registers and spilled; out of line it needs
-// none, and decoding is 4-26% faster across the codes, most for the
-// loop-bound eBCH(64,51)).  Same steps as the general loop in siso_word
-// below: chunks of 32 queries, each lane's next entry copied ahead by
-// cp.async, syndromes and double-float masses of the patterns, hits kept in
-// query order until L codewords are listed or the cap is reached.
-struct LoopOut {
-  int q, nhit, wacc;
-  DF tmass;
+// Record list words l0 .. l1 - 1 of a search from their query indices (lane l
+// holds hq of list word l): the codeword y + z in bit order (sc.cw()) and
+// log p(z)/p(0) = -sum |lambda| over z (sc.lp()).  Two words at a time, 16
+// lanes each: lane k of a half takes the pattern's k-th rank from the order
+// table `ent` (one byte load; lane 15 the weight).  Without the threshold
+// rule the list is recorded once, after the search.  The sum's butterfly adds
+// the same values in the same order as one over 32 lanes whose upper half
+// holds zeros.
+template <int NPL, class SYN>
+__device__ __forceinline__ void record_list(const Scratch<NPL, SYN> &sc, const uint4 *ent, int hq, int l0, int l1,
+                                            int lane) {
+  constexpr int NM = (32 * NPL + 63) / 64;
+  const int k = lane & 15;
+  int l = l0 + (lane >> 4);
+  const auto load = [&]() {  // list word l's byte of this lane
+    const int q = __shfl_sync(FULL, hq, l & 31);
+    return l < l1 ? (int)__ldg(reinterpret_cast<const uint8_t *>(ent + q) + ((k + 1) & 15)) : 0;
+  };
+  int nxt = load();
+  const int xw = lane & (2 * NM - 1);
+  const unsigned yw = xw < NPL ? sc.head_at(xw) : 0u;  // this lane's word of y
+#pragma unroll
+  for (int i = lane; i < LMAX * 2 * NM; i += 32)
+    if (i >= l0 * 2 * NM && i < l1 * 2 * NM) sc.cw32()[i] = yw;
+  __syncwarp();
+#pragma unroll 1
+  for (; l0 < l1; l0 += 2) {
+    const int at = l, v = nxt;
+    l += 2;
+    nxt = load();
+    const int w = __shfl_sync(FULL, v, lane | 15);  // 0 past the list
+    RankBit rb = {0.f, 0};
+    if (k < w) {
+      rb = sc.rb()[v];
+      atomicXor(sc.cw32() + at * 2 * NM + (rb.bit >> 5), 1u << (rb.bit & 31));
+    }
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) rb.a += __shfl_xor_sync(FULL, rb.a, d);
+    if (k == 0 && at < l1) sc.lp()[at] = -rb.a;
+  }
+  __syncwarp();
+}
+
+// ----------------------------------------------------------------------------
+// the search
+// ----------------------------------------------------------------------------
+// Chunks of 32 queries, lane j testing query q0 + j; hits are taken in query
+// order until L codewords are listed, the cap is reached or the threshold rule
+// applies.
+//
+// Prefix records.  A pattern of weight w costs a byte extract, a record load,
+// an XOR and a three-operation product for every rank.  In 1-line ORBGRAND
+// order the patterns of many consecutive queries share their low ranks:
+// without its last two ranks, the first thousand queries' patterns have only
+// 32 different prefixes, and without the last three the first nine thousand
+// have 64.  So the word first computes each prefix's record {syndrome of y XOR
+// its H columns, mass in double-float, weight} once, one lane each, and then
+// every query costs one 16-byte record, two (three) rank records and one
+// compact 4-byte entry {slot, ranks}, read a chunk ahead into a register (the
+// 16-byte entries cost four times the L2 traffic).  The factors are multiplied
+// in the same ascending order, so masses are bit for bit those of the
+// rank-by-rank product.  A word starts in the two-rank form (one 32-lane build
+// step), goes on in the three-rank form (two build steps), and past that, and
+// for a last partial chunk, tests the 16-byte entries rank by rank
+// (ent_syndrome).  64-bit syndromes leave no room for the record in 16 bytes
+// and always take the last form.
+
+// Where the query loop takes its patterns and when it stops.
+enum : int {
+  MODE_TABLE = 0,  // the order tables, no threshold rule
+  MODE_LANES = 1,  // enumerated by the lanes (DevCode::ord_lanes), no threshold rule
+  MODE_THR = 2     // the order tables, the threshold rule asked at every listed word
 };
-template <int NPL, class SYN>
-__device__ __noinline__ LoopOut query_loop_plain(const Scratch<NPL, SYN> sc, const WordHead<NPL, SYN> &h,
-                                                 const uint4 *ent, int qlim, int L, int lane) {
-  int q = 0, nhit = 0, wacc = 0;
-  DF tmass = {0.f, 0.f};
-#ifdef SG_PHASE_PROFILE
-  int nchunks = 0;
-#endif
-  const unsigned pf_addr = (unsigned)__cvta_generic_to_shared(sc.pf() + lane);
-  if (lane < qlim) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(pf_addr), "l"(ent + lane) : "memory");
-  asm volatile("cp.async.commit_group;" ::: "memory");
-  for (;;) {
-    const int lim = min(32, qlim - q);
-    if (lim <= 0) break;
-#ifdef SG_PHASE_PROFILE
-    nchunks++;
-#endif
-    uint4 e = make_uint4(0u, 0u, 0u, 0u);
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    if (lane < lim) e = sc.pf()[lane];
-    if (q + 32 + lane < qlim)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(pf_addr), "l"(ent + q + 32 + lane) : "memory");
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    const int w = e.x & 0xff;
-    const int wmax = (int)__reduce_max_sync(FULL, (unsigned)w);
-    DF mass;
-    const SYN s = ent_syndrome<SYN>(e, w, wmax, sc.hr(), mass) ^ h.s0;
-    const bool hit = lane < lim && s == 0;
-    unsigned hm = __ballot_sync(FULL, hit);
-    int stop_lane = -1;
-    while (hm) {
-      const int hl = __ffs(hm) - 1;
-      hm &= hm - 1;
-      record_hit<NPL, SYN>(sc, h, e, hl, nhit, lane);
-      nhit++;
-      if (nhit >= L) {
-        stop_lane = hl;
-        break;
-      }
-    }
-    if (stop_lane >= 0) {
-      if (lane <= stop_lane) {
-        wacc += w;
-        df_acc(tmass, mass);
-      }
-      q += stop_lane + 1;
-      break;
-    }
-    wacc += w;
-    df_acc(tmass, mass);
-    q += lim;
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-#ifdef SG_PHASE_PROFILE
-  if (lane == 0) SG_PROF(5, nchunks);
-#endif
-  return LoopOut{q, nhit, wacc, tmass};
-}
 
-// The thr = 0 query loop with the order enumerated by the lanes: the same
-// chunks of 32 queries, syndromes, masses and hit recording as
-// query_loop_plain; lane j finds the group of query q0 + j from the group
-// starts of the chunk (one coalesced load of the next 32 group records, a
-// bit mask of the groups that start inside the chunk) and unranks its offset
-// in that group.  The order's groups are grp[g0 .. ge - 1]; the arguments are
-// plain values and pointers (a reference to the kernel's code parameter would
-// make the compiler copy the parameter to local memory).
+// Compute the records of `count` prefix slots.
 template <int NPL, class SYN>
-__device__ __noinline__ LoopOut query_loop_lanes(const Scratch<NPL, SYN> sc, const WordHead<NPL, SYN> &h,
-                                                 const uint2 *grp, int g0, int ge, const int32_t *scnt, int sc_w,
-                                                 int sc_m, int n, int qlim, int L, int lane) {
-  int q = 0, nhit = 0, wacc = 0;
-  DF tmass = {0.f, 0.f};
-  GroupWindow W;
-  W.init(grp, g0, ge);
-  uint4 *slot = sc.pf() + lane;
-  for (;;) {
-    const int lim = min(32, qlim - q);
-    if (lim <= 0) break;
-    const uint4 e = W.chunk(q, lim, lane, scnt, sc_w, sc_m, n, slot);
-    const int w = e.x & 0xff;
-    const int wmax = (int)__reduce_max_sync(FULL, (unsigned)w);
-    DF mass;
-    const SYN s = ent_syndrome<SYN>(e, w, wmax, sc.hr(), mass) ^ h.s0;
-    const bool hit = lane < lim && s == 0;
-    unsigned hm = __ballot_sync(FULL, hit);
-    int stop_lane = -1;
-    while (hm) {
-      const int hl = __ffs(hm) - 1;
-      hm &= hm - 1;
-      record_hit<NPL, SYN>(sc, h, e, hl, nhit, lane);
-      nhit++;
-      if (nhit >= L) {
-        stop_lane = hl;
-        break;
+__device__ __forceinline__ void build_prefixes(const Scratch<NPL, SYN> &sc, SYN s0, const uint2 *slots, int count,
+                                               int lane) {
+  __syncwarp();  // every lane is done with the previous records
+#pragma unroll 1
+  for (int i0 = 0; i0 < count; i0 += 32) {  // count is a multiple of 32
+    uint2 d = __ldg(slots + i0 + lane);
+    const int len = d.x & 15, w = len + ((d.x >> 4) & 15);
+    const int longest = (int)__reduce_max_sync(FULL, (unsigned)len);
+    unsigned h = (unsigned)s0;
+    float mh = w > 0 ? 1.f : 0.f, ml = 0.f;  // the zero pattern has no queried mass
+#pragma unroll 1
+    for (int k = 0; k < longest; k++) {
+      d.x = __funnelshift_r(d.x, d.y, 8);
+      d.y >>= 8;
+      if (k < len) {
+        const RankRec<SYN> v = sc.hr()[d.x & 0xff];
+        h ^= (unsigned)v.h;
+        const float p = __fmul_rn(mh, v.t);
+        ml = fmaf(ml, v.t, fmaf(mh, v.t, -p));
+        mh = p;
       }
     }
-    if (stop_lane >= 0) {
-      if (lane <= stop_lane) {
-        wacc += w;
-        df_acc(tmass, mass);
-      }
-      q += stop_lane + 1;
-      break;
-    }
-    wacc += w;
-    df_acc(tmass, mass);
-    q += lim;
+    sc.prec()[i0 + lane] = make_uint4(h, __float_as_uint(mh), __float_as_uint(ml), (unsigned)w);
   }
-  return LoopOut{q, nhit, wacc, tmass};
-}
-
-// The thr = 0 query loop of a word: patterns from the order table, or
-// enumerated by the lanes (LANES, kernels of their own).
-template <int NPL, class SYN, bool LANES>
-__device__ __forceinline__ LoopOut query_loop(const Scratch<NPL, SYN> &sc, const WordHead<NPL, SYN> &h,
-                                              const DevCode &code, int ti, int tb, int qlim, int L, int lane) {
-  if constexpr (LANES)
-    return query_loop_lanes<NPL, SYN>(sc, h, code.grp.grp, __ldg(code.grp.gbase + ti), __ldg(code.grp.gbase + ti + 1),
-                                      code.grp.scnt, code.grp.sc_w, code.grp.sc_m, code.n, qlim, L, lane);
-  else
-    return query_loop_plain<NPL, SYN>(sc, h, code.ord.ent + tb, qlim, L, lane);
+  __syncwarp();
 }
 
 // lam[k] is bit lane + 32k of the SISO input lambda = fl32(L_Ch + L_A)
-// (the caller loads it; entries past n are ignored).  On return lapp[k] holds
-// L_APP for the same bits, res the per-word results; the list (in query
-// order) is left in the scratch: sc.cw() (codewords, natural bit order),
-// sc.lp() (log p(z)/p(0)) and sc.wl() (APP of each word).  *flags (if given)
-// collects the remaining-mass flags (bit 0: extended range; bit 1: the
-// block's remaining-mass area could not be locked).
-template <int NPL, class SYN, bool LANES = false>
-__device__ void siso_word(const DevCode &code, const SisoParams &P, const Scratch<NPL, SYN> &sc,
-                          const float (&lam)[NPL], int lane, float (&lapp)[NPL], WordResult &res,
-                          int *flags = nullptr) {
-  constexpr int NT = 32 * NPL;
-  constexpr int NM = (NT + 63) / 64;
+// (the caller loads it; entries past n are ignored).  L_APP is handed to
+// emit(k, x, lapp, listed) for k = 0 .. NPL - 1 in turn: bit lane + 32k, its
+// lambda x and whether the word's list holds a word (else lapp = x).  res gets
+// the per-word results (before the first emit); the list (in query order) is
+// left in the scratch: sc.cw() (codewords, natural bit order), sc.lp() (log
+// p(z)/p(0)) and sc.wl() (APP of each word).  res.flags collects
+// the remaining-mass flags (bit 0: extended range; bit 1: the block's
+// remaining-mass area could not be locked).
+//
+// What bounds a word is instruction fetch and issue: a word runs about two
+// thousand instructions once each around a short query loop, and the warps of
+// an SM are in different phases of their words, so the whole word's code
+// competes for the SM's instruction cache.  Everything that runs once per word
+// is therefore written for few instructions: lanes share what a single lane
+// could do (list words' APPs, candidates of the 1-line parameter), and loops
+// over the list and over a lane's bits stay rolled.
+template <int NPL, class SYN, int MODE, class Emit>
+__device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams &P, const Scratch<NPL, SYN> &sc,
+                                          const float (&lam)[NPL], int lane, WordResult &res, Emit emit) {
+  constexpr int NM = (32 * NPL + 63) / 64;
   const int n = code.n;
 #ifdef SG_PHASE_PROFILE
   const long long t0 = clock64();
@@ -1334,22 +1255,22 @@ __device__ void siso_word(const DevCode &code, const SisoParams &P, const Scratc
 #pragma unroll
   for (int k = 0; k < NPL; k++) sc.lamv()[lane + 32 * k] = lam[k];  // each lane reads back its own
   WordHead<NPL, SYN> h;
+  res.flags = res.wsum = res.nhit = 0;
+  res.queries = -1;
+  res.pmiss = 1.f;
   if (!siso_prologue<NPL, SYN>(code, sc, lam, lane, h)) {
-#pragma unroll
-    for (int k = 0; k < NPL; k++) lapp[k] = lam[k];
-    res.queries = -1;
-    res.nhit = 0;
-    res.pmiss = 1.f;
-    res.logD = 0.f;
-    res.wsum = 0;
+#pragma unroll 1
+    for (int k = 0; k < NPL; k++) {
+      const float x = sc.lam_at(lane + 32 * k);
+      emit(k, x, x, false);
+    }
     return;
   }
 #ifdef SG_PHASE_PROFILE
   const long long t1 = clock64();
-  int nchunks = 0;
 #endif
 
-  // query loop over the flattened order of (c, class)
+  // the order of (c, class)
   const DevOrder &O = code.ord;
   const int cls = code.even ? h.par : -1;
   const int ti = h.c * O.ncls + (code.even ? h.par : 0);
@@ -1357,157 +1278,206 @@ __device__ void siso_word(const DevCode &code, const SisoParams &P, const Scratc
 #pragma unroll
     for (int k = 0; k < NPL; k++) sc.headv()[k] = h.yb[k];
     sc.headv()[NPL] = (unsigned)h.c;
+    if (MODE == MODE_THR) sc.headv()[NPL + 1] = 0u;  // the class total is not known yet
   }
   __syncwarp();
   const int tb = __ldg(O.base + ti), tc = __ldg(O.count + ti);
   const int qlim = min(P.cap, tc);
-  int q = 0, nhit = 0;
-  float lr2 = 0.f;  // log2 remaining mass (set when the search stops)
-  bool have_lr2 = false;
-  int wacc = 0;       // this lane's share of the summed pattern weights
-  DF tmass = {0.f, 0.f};  // this lane's share of the queried mass (nonzero patterns)
-  // each lane's entry of the next chunk is copied into its 16-byte slot of the
-  // warp's shared area while the current chunk is tested (cp.async: no
-  // registers held, the L2 latency overlaps the chunk's work)
-  if (P.thr <= 0.f) {  // no threshold rule: the out-of-line loop
-    const LoopOut lo = query_loop<NPL, SYN, LANES>(sc, h, code, ti, tb, qlim, P.L, lane);
-    q = lo.q;
-    nhit = lo.nhit;
-    wacc = lo.wacc;
-    tmass = lo.tmass;
-  } else {  // with the threshold rule checked at every new list word
-    const unsigned pf_addr = (unsigned)__cvta_generic_to_shared(sc.pf() + lane);
-    if (lane < qlim)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(pf_addr), "l"(O.ent + tb + lane) : "memory");
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    for (;;) {
-      const int lim = min(32, qlim - q);
-      if (lim <= 0) break;
+  const uint4 *ent = O.ent + tb;
+
+  int q = 0, nhit = 0;    // the chunk's first query, the list
+  int hq = 0;             // lane l: the query index of list word l
+  int wacc = 0;           // this lane's share of the summed pattern weights
+  DF tmass = {0.f, 0.f};  // and of the queried mass (nonzero patterns)
+  GroupWindow win;
+  if constexpr (MODE == MODE_LANES)
+    win.init(code.grp.grp, __ldg(code.grp.gbase + ti), __ldg(code.grp.gbase + ti + 1));
+  // zone 0: two-rank form, 1: three-rank form, 2: 16-byte entries (or the lanes' patterns), 3: the end
+  int zone = -1, qe = 0;
+  unsigned hm = 0;   // the current chunk's hits still to take
+  int lim = 32, w = 0;
+  DF mass = {0.f, 0.f};
+  const uint32_t *e4 = O.e4 + (size_t)ti * O.e4_stride + lane;
+  unsigned e = 0;
+  int listed = 0;  // list words recorded so far
+  float M;         // log (R phi), natural
 #ifdef SG_PHASE_PROFILE
-      nchunks++;
+  long long t2 = 0;
 #endif
-      uint4 e = make_uint4(0u, 0u, 0u, 0u);
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      if (lane < lim) e = sc.pf()[lane];  // after the wait (a compiler barrier): this lane's own slot
-      if (q + 32 + lane < qlim)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(pf_addr), "l"(O.ent + tb + q + 32 + lane) : "memory");
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      const int w = e.x & 0xff;
-      const int wmax = (int)__reduce_max_sync(FULL, (unsigned)w);
-      DF mass;
-      const SYN s = ent_syndrome<SYN>(e, w, wmax, sc.hr(), mass) ^ h.s0;
-      const bool hit = lane < lim && s == 0;
-      unsigned hm = __ballot_sync(FULL, hit);
-      int stop_lane = -1;
-      while (hm) {
-        const int hl = __ffs(hm) - 1;
-        hm &= hm - 1;
-        record_hit<NPL, SYN>(sc, h, e, hl, nhit, lane);
-        nhit++;
-        if (nhit >= P.L) {
-          stop_lane = hl;
-          break;
+#pragma unroll 1
+  for (;;) {
+    // the search proper: to the hit that completes the list (MODE_THR: to the
+    // next hit), or to the end
+    int hl = -1;
+    bool fin = true;
+#pragma unroll 1
+    for (;;) {
+      if (hm == 0) {
+        // on to the next chunk with a hit, if any
+        if (q >= qe) {
+          zone++;
+          if (zone >= 3) break;  // the order or the cap ends here
+          lim = 32;
+          qe = qlim;
+          if (zone < 2) {
+            qe = 0;
+            if constexpr (MODE != MODE_LANES && sizeof(SYN) == 4) {
+              const int2 z = __ldg(O.zones + ti);
+              qe = min(zone ? z.y : z.x, qlim & ~31);
+              if (q < qe) {
+                e = __ldg(e4 + q);
+                build_prefixes<NPL, SYN>(sc, h.s0, O.slots + ti * (FAST_SLOTS2 + FAST_SLOTS) + (zone ? FAST_SLOTS2 : 0),
+                                         zone ? FAST_SLOTS : FAST_SLOTS2, lane);
+              }
+            }
+          }
+          continue;
         }
-        if (P.thr > 0.f) {
-          DF part = tmass;
-          if (lane <= hl) df_acc(part, mass);
-          const DF tq = df_warp_sum(part);
-          const float r2 = remaining_log2<NPL, SYN>(sc, O, tb, tc, q + hl, n, (int)sc.head_at(NPL), cls, lane, tq, flags);
-          if (thr_reached(sc, nhit, r2 * LN2_F + code.log_phi, P.thr)) {
-            stop_lane = hl;
-            lr2 = r2;
-            have_lr2 = true;
-            break;
+        if (MODE != MODE_LANES && sizeof(SYN) == 4 && zone < 2) {
+          // full chunks in the two- or three-rank form: one loop for both, so
+          // that its instructions are fetched once
+          const bool three = zone != 0;
+#pragma unroll 1
+          for (;;) {
+            const unsigned cur = e;
+            e = __ldg(e4 + q + 32);  // the table is padded by a chunk
+            const uint4 r = sc.prec()[cur & 0xff];
+            const RankRec<SYN> ra = sc.hr()[(cur >> 8) & 0xff], rb = sc.hr()[(cur >> 16) & 0xff];
+            unsigned s = r.x ^ (unsigned)ra.h ^ (unsigned)rb.h;
+            w = (int)r.w;
+            mass = DF{__uint_as_float(r.y), __uint_as_float(r.z)};
+            const auto mul = [&](float t) {
+              const float p = __fmul_rn(mass.h, t);
+              mass.l = fmaf(mass.l, t, fmaf(mass.h, t, -p));
+              mass.h = p;
+            };
+            mul(ra.t);
+            mul(rb.t);
+            if (three) {
+              const RankRec<SYN> rc = sc.hr()[cur >> 24];
+              s ^= (unsigned)rc.h;
+              mul(rc.t);
+            }
+            hm = __ballot_sync(FULL, s == 0);
+            if (hm != 0) break;
+            wacc += w;
+            df_acc(tmass, mass);
+            q += 32;
+            if (q >= qe) break;
+          }
+        } else {
+          // one chunk rank by rank
+          lim = min(32, qlim - q);
+          uint4 ee = make_uint4(0u, 0u, 0u, 0u);
+          if constexpr (MODE == MODE_LANES) {
+            ee = win.chunk(q, lim, lane, code.grp.scnt, code.grp.sc_w, code.grp.sc_m, n, sc.pf() + lane);
+          } else {
+            if (lane < lim) ee = __ldg(ent + q + lane);
+          }
+          w = ee.x & 0xff;
+          const int wmax = (int)__reduce_max_sync(FULL, (unsigned)w);
+          const SYN s = ent_syndrome<SYN>(ee, w, wmax, sc.hr(), mass) ^ h.s0;
+          hm = __ballot_sync(FULL, lane < lim && s == 0);
+          if (hm == 0) {  // lanes past lim hold an empty entry
+            wacc += w;
+            df_acc(tmass, mass);
+            q += lim;
           }
         }
+        if (hm == 0) continue;
       }
-      if (stop_lane >= 0) {
-        if (lane <= stop_lane) {
-          wacc += w;
-          df_acc(tmass, mass);
-        }
-        q += stop_lane + 1;
-        break;
+      // the chunk's next hit
+      hl = __ffs(hm) - 1;
+      hm &= hm - 1;
+      if (lane == nhit) hq = q + hl;
+      nhit++;
+      fin = nhit >= P.L;
+      if (MODE == MODE_THR || fin) break;
+      hl = -1;
+      if (hm == 0) {
+        wacc += w;
+        df_acc(tmass, mass);
+        q += lim;
       }
-      wacc += w;  // lanes past lim hold an empty entry
+    }
+#ifdef SG_PHASE_PROFILE
+    if (t2 == 0) t2 = clock64();
+#endif
+    record_list<NPL, SYN>(sc, ent, hq, listed, nhit, lane);
+    listed = nhit;
+    // the queries made up to here: qn, their mass `part`
+    const int qn = hl >= 0 ? q + hl + 1 : q;
+    DF part = tmass;
+    if (lane <= hl) df_acc(part, mass);
+    Remaining rem = {-CUDART_INF_F, 0};
+    // when the whole parity class has been queried nothing remains
+    if (!(fin && qn >= tc && tc == O.class_size) && !P.forney)
+      rem = remaining_log2<MODE == MODE_THR, NPL, SYN>(sc, ent, O.cost + tb, tc, qn - 1, n, cls, lane,
+                                                       df_warp_sum(part));
+    res.flags |= rem.flags;
+    M = fmaf(rem.lr2, LN2_F, code.log_phi);
+    if (MODE != MODE_THR || fin || thr_reached(sc.lp(), nhit, M, P.thr)) {
+      if (lane <= hl) wacc += w;
+      q = qn;
+      break;
+    }
+    if (hm == 0) {  // that was the chunk's last hit
+      wacc += w;
       df_acc(tmass, mass);
       q += lim;
     }
-    // a copy for a chunk that was not needed may still be in flight: wait for
-    // it, so that it cannot land in the slot after the next word's first copy
-    asm volatile("cp.async.wait_all;" ::: "memory");
   }
-  // the whole parity class has been queried: nothing remains
-  const bool exhausted = q >= tc && tc == O.class_size;
-  __syncwarp();
 #ifdef SG_PHASE_PROFILE
-  const long long t2 = clock64();
-#endif
-
-  // soft output (Corollary + eq. LLRi)
-  if (!have_lr2)
-    lr2 = (exhausted || P.forney) ? -CUDART_INF_F
-                    : remaining_log2<NPL, SYN>(sc, O, tb, tc, q - 1, n, (int)sc.head_at(NPL), cls, lane, df_warp_sum(tmass),
-                                               flags);
-#ifdef SG_PHASE_PROFILE
+  if (lane == 0) SG_PROF(5, (q + 31) / 32);
   const long long t3 = clock64();
 #endif
-  const float M = lr2 * LN2_F + code.log_phi;  // log (R phi), natural
   res.wsum = (int32_t)__reduce_add_sync(FULL, (unsigned)wacc);
   res.queries = q;
   res.nhit = nhit;
-  if (nhit == 0) {
-#pragma unroll
-    for (int k = 0; k < NPL; k++) lapp[k] = sc.lam_at(lane + 32 * k);
-    res.pmiss = 1.f;
-    res.logD = M;
-  } else {
-    // log(R phi + sum_l p_l), all relative to p(0): max plus log of a sum.
-    // The hardware exponential and logarithm (relative errors near 2^-21 over
-    // these ranges) keep L_APP within about 1e-5 of the exact formula, far
-    // inside the soft output's tolerance; no decision is taken on them.
-    float mx = M;
-    for (int l = 0; l < nhit; l++) mx = fmaxf(mx, sc.lp()[l]);
-    float sum = M == -CUDART_INF_F ? 0.f : __expf(M - mx);
-    for (int l = 0; l < nhit; l++) sum += __expf(sc.lp()[l] - mx);
-    const float D = mx + __logf(sum);
-    res.logD = D;
-    const float pm = M == -CUDART_INF_F ? 0.f : __expf(M - D);
-    res.pmiss = pm;
-    // APP of each listed word (list weights relative to the normaliser)
-    if (lane < nhit) sc.wl()[lane] = __expf(sc.lp()[lane] - D);
-    __syncwarp();
-    // eq. LLRi: the miss term, then each listed word adds its APP to the side
-    // of its bit; a list word's bit mask is read once for all the lane's bits
-    float a0[NPL], a1[NPL];
-#pragma unroll
-    for (int k = 0; k < NPL; k++) {
-      const float x = sc.lam_at(lane + 32 * k);
-      // sigma(x) and sigma(-x) without cancellation
-      const float ex = __expf(-fabsf(x));
-      const float sp = __fdividef(1.f, 1.f + ex), sn = ex * sp;  // sigma(|x|), sigma(-|x|)
-      a0[k] = pm * (x >= 0.f ? sp : sn);                          // miss term, bit 0
-      a1[k] = pm * (x >= 0.f ? sn : sp);                          // miss term, bit 1
-    }
+  // log(R phi + sum_l p_l), all relative to p(0): max plus log of a sum
+  // (lane l takes list word l; the terms are added in list order).  The
+  // hardware exponential and logarithm (relative errors near 2^-21 over
+  // these ranges) keep L_APP within about 1e-5 of the exact formula, far
+  // inside the soft output's tolerance; no decision is taken on them.
+  const float lp = lane < nhit ? sc.lp()[lane] : -CUDART_INF_F;
+  // log masses are <= 0: the largest has the smallest magnitude bits
+  const float mx = fmaxf(M, -__uint_as_float(__reduce_min_sync(FULL, __float_as_uint(-lp) & 0x7fffffffu)));
+  float sum = M == -CUDART_INF_F ? 0.f : __expf(M - mx);
+  const float el = __expf(lp - mx);
+#pragma unroll 1
+  for (int l = 0; l < nhit; l++) sum += __shfl_sync(FULL, el, l);
+  const float D = mx + __logf(sum);
+  const float pm = M == -CUDART_INF_F ? 0.f : __expf(M - D);
+  if (nhit > 0) res.pmiss = pm;
+  // APP of each listed word (list weights relative to the normaliser)
+  const float wl = __expf(lp - D);
+  if (lane < nhit) sc.wl()[lane] = wl;
+  // eq. LLRi: the miss term, then each listed word adds its APP to the side
+  // of its bit
+#pragma unroll 1
+  for (int k = 0; k < NPL; k++) {
+    const float x = sc.lam_at(lane + 32 * k);
+    // sigma(x) and sigma(-x) without cancellation
+    const float ex = __expf(-fabsf(x));
+    const float sp = __fdividef(1.f, 1.f + ex), sn = ex * sp;  // sigma(|x|), sigma(-|x|)
+    float a0 = pm * (x >= 0.f ? sp : sn);                       // miss term, bit 0
+    float a1 = pm * (x >= 0.f ? sn : sp);                       // miss term, bit 1
+#pragma unroll 1
     for (int l = 0; l < nhit; l++) {
-      const float wlv = sc.wl()[l];
-#pragma unroll
-      for (int k = 0; k < NPL; k++) {
-        const int i = lane + 32 * k;
-        if ((sc.cw()[l * NM + (i >> 6)] >> (i & 63)) & 1ull)
-          a1[k] += wlv;
-        else
-          a0[k] += wlv;
-      }
+      const float wlv = __shfl_sync(FULL, wl, l);
+      if ((sc.cw32()[l * 2 * NM + k] >> lane) & 1u)
+        a1 += wlv;
+      else
+        a0 += wlv;
     }
-#pragma unroll
-    for (int k = 0; k < NPL; k++) {
-      // both sums lie in (1e-30, 1 + 1e-6]: __fdividef's range
-      lapp[k] = (a0[k] > 1e-30f && a1[k] > 1e-30f)
-                    ? __logf(__fdividef(a0[k], a1[k]))
-                    : lapp_logdomain<NPL, SYN>(sc, nhit, M, sc.lam_at(lane + 32 * k), lane + 32 * k);
-    }
+    // both sums lie in (1e-30, 1 + 1e-6]: __fdividef's range
+    float lapp = x;
+    if (nhit > 0)
+      lapp = (a0 > 1e-30f && a1 > 1e-30f) ? __logf(__fdividef(a0, a1))
+                                          : lapp_logdomain<NPL, SYN>(sc, nhit, M, x, lane + 32 * k);
+    emit(k, x, lapp, nhit > 0);
   }
+  __syncwarp();
 #ifdef SG_PHASE_PROFILE
   const long long t4 = clock64();
   if (lane == 0) {
@@ -1516,7 +1486,6 @@ __device__ void siso_word(const DevCode &code, const SisoParams &P, const Scratc
     SG_PROF(2, t3 - t2);
     SG_PROF(3, t4 - t3);
     SG_PROF(4, 1);
-    SG_PROF(5, nchunks);
   }
 #endif
 }
