@@ -76,7 +76,7 @@ struct HostTables {
   std::vector<int32_t> scnt;    // [N = 0..n][w < sc_w][m < sc_m]
   int sc_w = 1, sc_m = 1;
   // the head of every order as prefix slot + last ranks (DevOrder::e4)
-  std::vector<uint32_t> e4;
+  std::vector<uint4> e4;
   std::vector<uint2> slots;
   std::vector<int2> zones;
   int e4_stride = 0;
@@ -85,7 +85,8 @@ struct HostTables {
 // One zone of an order's compact form: entries from `q` on as a prefix slot
 // and the last `ranks` ranks, slots assigned in order of first use, until
 // another slot would be needed, a prefix would not fit its descriptor, or the
-// entries kept end.  The zone stops at a whole chunk.  Returns its end.
+// entries kept end.  The zone stops at a whole group of four chunks.  Returns
+// its end.
 int compact_zone(const uint4 *ent, int q, int count, int n, int ranks, int max_slots, uint2 *slots,
                  std::vector<uint32_t> &out) {
   // open-addressed table of the slots in use, keyed by their descriptor
@@ -113,7 +114,7 @@ int compact_zone(const uint4 *ent, int q, int count, int n, int ranks, int max_s
     for (int i = 0; i < 3; i++) e |= (uint32_t)(i < rest ? b[1 + len + i] : n) << (8 + 8 * i);
     out.push_back(e);
   }
-  const int end = start + ((q - start) & ~31);
+  const int end = start + ((q - start) & ~127);
   out.resize(out.size() - (size_t)(q - end));
   return end;
 }
@@ -255,10 +256,13 @@ int build_tables(int n, int64_t cap, int c_max, bool even, HostTables &T) {
     z.y = compact_zone(ent, z.x, count, n, 3, sg::FAST_SLOTS, &T.slots[(size_t)ti * per + sg::FAST_SLOTS2], heads[ti]);
     longest = std::max(longest, z.y);
   }
-  T.e4_stride = longest + 64;  // padded: a chunk past the head is read ahead
-  T.e4.assign((size_t)orders * T.e4_stride, 0u);
-  for (int ti = 0; ti < orders; ti++)
-    std::copy(heads[ti].begin(), heads[ti].end(), T.e4.begin() + (size_t)ti * T.e4_stride);
+  T.e4_stride = longest / 4 + 64;  // padded: two groups past the head are read ahead
+  T.e4.assign((size_t)orders * T.e4_stride, make_uint4(0u, 0u, 0u, 0u));
+  for (int ti = 0; ti < orders; ti++) {
+    uint32_t *dst = &T.e4[(size_t)ti * T.e4_stride].x;
+    for (size_t q = 0; q < heads[ti].size(); q++)  // query 128 g + 32 c + j: lane j's c-th entry of group g
+      dst[(q & ~size_t(127)) + 4 * (q & 31) + ((q >> 5) & 3)] = heads[ti][q];
+  }
   T.jmax = maxcost + 2;
   T.gbase.push_back((int32_t)T.grp.size());
   // scnt[N][w][m]: w-subsets of {1..N} with sum m (N = 0..n, w < sc_w, m <= the
@@ -288,7 +292,7 @@ int upload_tables(sogrand_code *c, const HostTables &T, int64_t cap) {
   const size_t bi = T.base.size() * sizeof(int32_t);
   const size_t bg = T.grp.size() * sizeof(uint2), bgb = T.gbase.size() * sizeof(int32_t);
   const size_t bs = T.scnt.size() * sizeof(int32_t);
-  const size_t b4 = T.e4.size() * sizeof(uint32_t), bsl = T.slots.size() * sizeof(uint2);
+  const size_t b4 = T.e4.size() * sizeof(uint4), bsl = T.slots.size() * sizeof(uint2);
   const size_t bz = T.zones.size() * sizeof(int2);
   const size_t bytes = al(be) + al(bc) + 2 * al(bi) + al(bg) + al(bgb) + al(bs) + al(b4) + al(bsl) + al(bz);
   void *mem = nullptr;
@@ -301,7 +305,7 @@ int upload_tables(sogrand_code *c, const HostTables &T, int64_t cap) {
   uint2 *dgrp = (uint2 *)(p + al(be) + al(bc) + 2 * al(bi));
   int32_t *dgbase = (int32_t *)((char *)dgrp + al(bg));
   int32_t *dscnt = (int32_t *)((char *)dgbase + al(bgb));
-  uint32_t *de4 = (uint32_t *)((char *)dscnt + al(bs));
+  uint4 *de4 = (uint4 *)((char *)dscnt + al(bs));
   uint2 *dslots = (uint2 *)((char *)de4 + al(b4));
   int2 *dzones = (int2 *)((char *)dslots + al(bsl));
   if (cudaMemcpy(de4, T.e4.data(), b4, cudaMemcpyHostToDevice) != cudaSuccess ||

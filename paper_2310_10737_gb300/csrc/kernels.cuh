@@ -122,7 +122,8 @@ __global__ void __launch_bounds__(TPB, resident_blocks(MINB)) k_decode(const __g
       if (a.wsum) atomicAdd(a.wsum, (unsigned long long)res.wsum);
     }
     if (a.list_words || a.list_app) {
-      for (int l = lane; l < P.L; l += 32) {
+      const int l = lane;
+      if (l < P.L) {  // L <= 16
         if (a.list_words)
 #pragma unroll
           for (int wd = 0; wd < NM; wd++)
@@ -352,27 +353,20 @@ __device__ __forceinline__ bool frame_valid_diag(const DevCode &code, const uint
   constexpr int NM = (32 * NPL + 63) / 64;
   const int n = code.n;
   bool ok = true;
-#pragma unroll
-  for (int k = 0; k < NPL; k++) {
-    const int x = lane + 32 * k;
-    if (x < n) {
 #pragma unroll 1
-      for (int t = 0; t < code.m && ok; t++) {
-        int p = 0;
-#pragma unroll
-        for (int y = 0; y < NM; y++) p ^= __popcll(W[x * NM + y] & __ldg(code.hrow + t * NM + y));
-        if (p & 1) ok = false;
-      }
-      uint64_t syn = 0;
-      int w = x;  // (x + j) mod n after rows, (x - j) mod n after diagonals
+  for (int x0 = 0; x0 < n; x0 += 32) {
+    const int x = min(x0 + lane, n - 1);
+    uint64_t own = 0, other = 0;  // syndromes of word x and of word x of the other set
+    int w = x;                    // (x + j) mod n after rows, (x - j) mod n after diagonals
 #pragma unroll 1
-      for (int j = 0; j < n; j++) {
-        if ((W[w * NM + (j >> 6)] >> (j & 63)) & 1ull) syn ^= __ldg(code.hcol + j);
-        w += rows ? 1 : n - 1;
-        if (w >= n) w -= n;
-      }
-      if (syn) ok = false;
+    for (int j = 0; j < n; j++) {
+      const uint64_t h = __ldg(code.hcol + j);
+      if ((W[x * NM + (j >> 6)] >> (j & 63)) & 1ull) own ^= h;
+      if ((W[w * NM + (j >> 6)] >> (j & 63)) & 1ull) other ^= h;
+      w += rows ? 1 : n - 1;
+      if (w >= n) w -= n;
     }
+    ok = ok && (own | other) == 0;
   }
   return __all_sync(FULL, ok);
 }
@@ -416,27 +410,30 @@ __device__ __forceinline__ void frame_finish(const ProductArgs &a, int64_t f, bo
   }
   const bool aligned = (nr & 7) == 0 && !diag;
 #pragma unroll 1
-  for (int by = lane; by < nbytes; by += 32) {
+  for (int b0 = 0; b0 < nbytes; b0 += 32) {
+    const int by = min(b0 + lane, nbytes - 1);
     int i = by * 8 / nr, j = by * 8 - i * nr;
     unsigned v = 0;
     if (aligned) {
       v = Ws[i * W32 + (j >> 5)] >> (j & 31);
     } else {
 #pragma unroll 1
-      for (int t = 0; t < 8 && i < nc; t++) {
-        int w = i;
-        if (diag) {
-          w = i - j;
-          if (w < 0) w += nr;
+      for (int t = 0; t < 8; t++) {
+        if (i < nc) {
+          int w = i;
+          if (diag) {
+            w = i - j;
+            if (w < 0) w += nr;
+          }
+          v |= ((Ws[w * W32 + (j >> 5)] >> (j & 31)) & 1u) << t;
         }
-        v |= ((Ws[w * W32 + (j >> 5)] >> (j & 31)) & 1u) << t;
         if (++j == nr) {
           j = 0;
           i++;
         }
       }
     }
-    out[by] = (uint8_t)v;
+    if (b0 + lane < nbytes) out[by] = (uint8_t)v;
   }
   if (lane == 0) {
     a.half_iters[f] = half;
@@ -598,7 +595,8 @@ __device__ __forceinline__ void frame_after_half(const DevCode &wc, const DevCod
   __syncwarp();  // after lane 0's acquire of the frame's word count: the other words' results
   const uint64_t *hb = a.hb + (size_t)f * (GEN ? a.hbw : n) * NM;
 #pragma unroll 1
-  for (int x = lane; x < n * NM; x += 32) W[x] = ld_state<true>(hb + x);
+  for (int x0 = 0; x0 < n * NM; x0 += 32)
+    if (x0 + lane < n * NM) W[x0 + lane] = ld_state<true>(hb + x0 + lane);
   const int half = __ldcg(a.half_cur + f), bad = __ldcg(a.bad + f);
   const int stop = a.half_stop ? __ldcg(a.half_stop + f) : a.max_half;
   __syncwarp();

@@ -31,12 +31,17 @@ struct DevOrder {
   int32_t ncls;           // 2 for an even code (class = parity of y), else 1
   int32_t class_size;     // patterns in one class (saturated): count == class_size means the whole class
   // The head of every order again, a pattern as its prefix and its last ranks
-  // (see query_loop_plain): order (c, class) = ti owns e4[ti * e4_stride ...]
+  // (see siso_word's search): order (c, class) = ti owns e4[ti * e4_stride ...]
   // and slots[ti * (FAST_SLOTS2 + FAST_SLOTS) ...].
-  const uint32_t *e4;     // byte 0: prefix slot; bytes 1..3: the last ranks (0-based; n where there is none)
+  // e4: one 32-bit entry a query, byte 0: prefix slot; bytes 1..3: the last
+  // ranks (0-based; n where there is none).  Groups of four chunks, lane j's
+  // four entries together (uint4 [group][lane]): one load serves four chunks,
+  // and a warp alone on its SM, which waits out the L2 latency for every load,
+  // waits once in 128 queries.
+  const uint4 *e4;
   const uint2 *slots;     // byte 0: prefix length | ranks after it << 4; bytes 1..7: the prefix's ranks
-  const int2 *zones;      // [ti] queries in two-rank form (slots 0..31) and, from there, in three-rank form up to .y
-  int32_t e4_stride;
+  const int2 *zones;      // [ti] queries in two-rank form (slots 0..31) and, from there, in three-rank form up to .y (multiples of 128)
+  int32_t e4_stride;      // in uint4
 };
 
 // Prefix slots of the two-rank and the three-rank form, and the longest prefix.

@@ -310,23 +310,24 @@ struct Scratch {
 // spinning for ever: the warp then proceeds without the lock and reports it
 // (returns false).
 __device__ __forceinline__ bool dp_lock(int *lock, int lane) {
-  int ok = 1;
-  if (lane == 0) {
-    unsigned nap = 32;
-    long long tries = 0;
-    const long long limit = *reinterpret_cast<volatile int *>(lock + 1);
-    while (atomicCAS(lock, 0, 1) != 0) {
-      if (++tries > limit) {
-        ok = 0;
-        break;
-      }
-      __nanosleep(nap);
-      if (nap < 1024) nap <<= 1;
+  unsigned nap = 32;
+  long long tries = 0;
+  const long long limit = *reinterpret_cast<volatile int *>(lock + 1);
+  bool ok = true;
+#pragma unroll 1
+  for (;;) {
+    int got = 0;
+    if (lane == 0) got = atomicCAS(lock, 0, 1) == 0;
+    if (__shfl_sync(0xffffffffu, got, 0)) break;
+    if (++tries > limit) {
+      ok = false;
+      break;
     }
+    __nanosleep(nap);
+    if (nap < 1024) nap <<= 1;
   }
-  ok = __shfl_sync(0xffffffffu, ok, 0);
   __threadfence_block();
-  return ok != 0;
+  return ok;
 }
 __device__ __forceinline__ void dp_unlock(int *lock, bool held, int lane) {
   __syncwarp();
@@ -512,13 +513,16 @@ __device__ __forceinline__ void dp_ranks(int Cs, int c, int R0, int cls, const t
                                          typename Ops::T *ho, int lane, typename Ops::T &acc) {
   using T = typename Ops::T;
   constexpr bool SCALED = sizeof(T) == 4;
+  const int nslot = (Cs + 32) >> 5;
 #pragma unroll 1
-  for (int j = lane; j <= Cs; j += 32) {
-    he[j] = j == 0 ? Ops::one() : Ops::zero();
-    ho[j] = Ops::zero();
+  for (int t = 0; t < nslot; t++) {
+    const int j = 32 * t + lane;
+    if (j <= Cs) {
+      he[j] = j == 0 ? Ops::one() : Ops::zero();
+      ho[j] = Ops::zero();
+    }
   }
   __syncwarp();
-  const int nslot = (Cs + 32) >> 5;
   const bool ascending = SCALED && Cs < 128;
 #pragma unroll 1
   for (int e = 0; e <= R0; e++) {
@@ -660,16 +664,22 @@ __device__ __forceinline__ typename Ops::T remaining_scaled(const Scratch<NPL, S
     }
   }
   if constexpr (SCALED)
-    for (int j = lane; j <= Cs; j += 32) ek[j] = exp2f(-g2 * (float)j);
+#pragma unroll 1
+    for (int j0 = 0; j0 <= Cs; j0 += 32)
+      if (j0 + lane <= Cs) ek[j0 + lane] = exp2f(-g2 * (float)(j0 + lane));
   __syncwarp();
 
   // --- high ranks (d_e > Cs): G_P = sum_e sfac_e * F_{e+1} (parity of the
   //     pattern {e} + any higher subset), reduced over the warp
   T g_even = Ops::zero(), g_odd = Ops::zero();
-  for (int e = R0 + lane; e < n; e += 32) {
-    const T s = sfac[e];
-    g_odd = Ops::fma(s, Ops::add(Ops::one(), fu[e + 1]), g_odd);
-    g_even = Ops::fma(s, fb[e + 1], g_even);
+#pragma unroll 1
+  for (int e0 = R0; e0 < n; e0 += 32) {
+    const int e = e0 + lane;
+    if (e < n) {
+      const T s = sfac[e];
+      g_odd = Ops::fma(s, Ops::add(Ops::one(), fu[e + 1]), g_odd);
+      g_even = Ops::fma(s, fb[e + 1], g_even);
+    }
   }
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) {
@@ -761,7 +771,11 @@ __device__ __forceinline__ Remaining remaining_log2_dp(const Scratch<NPL, SYN> &
   const int Cs = __ldg(cost + qs);
   const int R0 = min(max(Cs - c, 0), n);
   float g = CUDART_INF_F;
-  for (int e = lane; e < R0; e += 32) g = fminf(g, sc.l2(e) / (float)(e + 1 + c));
+#pragma unroll 1
+  for (int e0 = 0; e0 < R0; e0 += 32) {
+    const int e = e0 + lane;
+    if (e < R0) g = fminf(g, sc.l2(e) / (float)(e + 1 + c));
+  }
   g = __shfl_sync(FULL, warp_min_f(g), 0);
   if (!(g < CUDART_INF_F)) g = 0.f;
   const bool held = dp_lock(sc.lock(), lane);
@@ -1237,6 +1251,11 @@ __device__ __forceinline__ void build_prefixes(const Scratch<NPL, SYN> &sc, SYN 
 // the remaining-mass flags (bit 0: extended range; bit 1: the block's
 // remaining-mass area could not be locked).
 //
+// Loops whose trip count differs between lanes are avoided throughout: after
+// one the compiler no longer knows the warp to be converged, and every later
+// shuffle and vote of the kernel pays for a check (about 135 instructions a
+// word when only the rarely run remaining-mass sums had such loops).
+//
 // What bounds a word is instruction fetch and issue: a word runs about two
 // thousand instructions once each around a short query loop, and the warps of
 // an SM are in different phases of their words, so the whole word's code
@@ -1294,11 +1313,27 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
     win.init(code.grp.grp, __ldg(code.grp.gbase + ti), __ldg(code.grp.gbase + ti + 1));
   // zone 0: two-rank form, 1: three-rank form, 2: 16-byte entries (or the lanes' patterns), 3: the end
   int zone = -1, qe = 0;
-  unsigned hm = 0;   // the current chunk's hits still to take
+  unsigned hm = 0;  // the current chunk's hits still to take
   int lim = 32, w = 0;
   DF mass = {0.f, 0.f};
-  const uint32_t *e4 = O.e4 + (size_t)ti * O.e4_stride + lane;
-  unsigned e = 0;
+  const uint4 *e4 = O.e4 + (size_t)ti * O.e4_stride + lane;
+  uint4 e = make_uint4(0u, 0u, 0u, 0u), en = e;  // this lane's entries of the current group of chunks and the next
+  // takes the chunk's hits in order: the lane of the one the search leaves at, or -1
+  const auto take = [&]() {
+    do {
+      const int at = __ffs(hm) - 1;
+      hm &= hm - 1;
+      if (lane == nhit) hq = q + at;
+      nhit++;
+      if (MODE == MODE_THR || nhit >= P.L) return at;
+    } while (hm != 0);
+    return -1;
+  };
+  const auto queried = [&]() {  // the whole chunk has been queried
+    wacc += w;
+    df_acc(tmass, mass);
+    q += lim;
+  };
   int listed = 0;  // list words recorded so far
   float M;         // log (R phi), natural
 #ifdef SG_PHASE_PROFILE
@@ -1309,100 +1344,105 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
     // the search proper: to the hit that completes the list (MODE_THR: to the
     // next hit), or to the end
     int hl = -1;
-    bool fin = true;
+    if (MODE == MODE_THR && hm != 0) {
+      hl = take();
+      goto left;
+    }
 #pragma unroll 1
     for (;;) {
-      if (hm == 0) {
-        // on to the next chunk with a hit, if any
-        if (q >= qe) {
-          zone++;
-          if (zone >= 3) break;  // the order or the cap ends here
-          lim = 32;
-          qe = qlim;
-          if (zone < 2) {
-            qe = 0;
-            if constexpr (MODE != MODE_LANES && sizeof(SYN) == 4) {
-              const int2 z = __ldg(O.zones + ti);
-              qe = min(zone ? z.y : z.x, qlim & ~31);
-              if (q < qe) {
-                e = __ldg(e4 + q);
-                build_prefixes<NPL, SYN>(sc, h.s0, O.slots + ti * (FAST_SLOTS2 + FAST_SLOTS) + (zone ? FAST_SLOTS2 : 0),
-                                         zone ? FAST_SLOTS : FAST_SLOTS2, lane);
-              }
+      if (q >= qe) {
+        zone++;
+        if (zone >= 3) break;
+        lim = 32;
+        qe = qlim;
+        if (MODE != MODE_LANES && zone == 2)
+          en = __ldg(ent + min(q + lane, tc - 1));
+        if (zone < 2) {
+          qe = 0;
+          if constexpr (MODE != MODE_LANES && sizeof(SYN) == 4) {
+            const int2 z = __ldg(O.zones + ti);
+            qe = min(zone ? z.y : z.x, qlim & ~127);
+            if (q < qe) {
+              e = __ldg(e4 + (q >> 2));
+              en = __ldg(e4 + (q >> 2) + 32);
+              build_prefixes<NPL, SYN>(sc, h.s0, O.slots + ti * (FAST_SLOTS2 + FAST_SLOTS) + (zone ? FAST_SLOTS2 : 0),
+                                       zone ? FAST_SLOTS : FAST_SLOTS2, lane);
             }
           }
-          continue;
         }
-        if (MODE != MODE_LANES && sizeof(SYN) == 4 && zone < 2) {
-          // full chunks in the two- or three-rank form: one loop for both, so
-          // that its instructions are fetched once
-          const bool three = zone != 0;
+      } else if (MODE != MODE_LANES && sizeof(SYN) == 4 && zone < 2) {
+        // full chunks in the two- or three-rank form: one loop for both, so
+        // that its instructions are fetched once
+        const bool three = zone != 0;
 #pragma unroll 1
-          for (;;) {
-            const unsigned cur = e;
-            e = __ldg(e4 + q + 32);  // the table is padded by a chunk
-            const uint4 r = sc.prec()[cur & 0xff];
-            const RankRec<SYN> ra = sc.hr()[(cur >> 8) & 0xff], rb = sc.hr()[(cur >> 16) & 0xff];
-            unsigned s = r.x ^ (unsigned)ra.h ^ (unsigned)rb.h;
-            w = (int)r.w;
-            mass = DF{__uint_as_float(r.y), __uint_as_float(r.z)};
-            const auto mul = [&](float t) {
-              const float p = __fmul_rn(mass.h, t);
-              mass.l = fmaf(mass.l, t, fmaf(mass.h, t, -p));
-              mass.h = p;
-            };
-            mul(ra.t);
-            mul(rb.t);
-            if (three) {
-              const RankRec<SYN> rc = sc.hr()[cur >> 24];
-              s ^= (unsigned)rc.h;
-              mul(rc.t);
-            }
-            hm = __ballot_sync(FULL, s == 0);
-            if (hm != 0) break;
-            wacc += w;
-            df_acc(tmass, mass);
-            q += 32;
-            if (q >= qe) break;
+        do {
+          const unsigned cur = e.x;
+          e.x = e.y;
+          e.y = e.z;
+          e.z = e.w;
+          if ((q & 96) == 96) {  // the group's last chunk
+            e = en;
+            en = __ldg(e4 + (q >> 2) + 40);  // q / 4 is 24 past the group; the table is padded by two groups
           }
-        } else {
-          // one chunk rank by rank
+          const uint4 r = sc.prec()[cur & 0xff];
+          const RankRec<SYN> ra = sc.hr()[(cur >> 8) & 0xff], rb = sc.hr()[(cur >> 16) & 0xff];
+          unsigned s = r.x ^ (unsigned)ra.h ^ (unsigned)rb.h;
+          w = (int)r.w;
+          mass = DF{__uint_as_float(r.y), __uint_as_float(r.z)};
+          const auto mul = [&](float t) {
+            const float p = __fmul_rn(mass.h, t);
+            mass.l = fmaf(mass.l, t, fmaf(mass.h, t, -p));
+            mass.h = p;
+          };
+          mul(ra.t);
+          mul(rb.t);
+          if (three) {
+            const RankRec<SYN> rc = sc.hr()[cur >> 24];
+            s ^= (unsigned)rc.h;
+            mul(rc.t);
+          }
+          hm = __ballot_sync(FULL, s == 0);
+          if (hm != 0) {
+            hl = take();
+            if (hl >= 0) goto left;
+          }
+          queried();
+        } while (q < qe);
+      } else {
+        // rank by rank, the entries read a chunk ahead
+#pragma unroll 1
+        do {
           lim = min(32, qlim - q);
-          uint4 ee = make_uint4(0u, 0u, 0u, 0u);
+          uint4 ee;
           if constexpr (MODE == MODE_LANES) {
             ee = win.chunk(q, lim, lane, code.grp.scnt, code.grp.sc_w, code.grp.sc_m, n, sc.pf() + lane);
           } else {
-            if (lane < lim) ee = __ldg(ent + q + lane);
+            // an empty entry past the end (selected, not branched to: a branch
+            // on the lane here costs the kernel its proof of convergence)
+            ee.x = lane < lim ? en.x : 0u;
+            ee.y = lane < lim ? en.y : 0u;
+            ee.z = lane < lim ? en.z : 0u;
+            ee.w = lane < lim ? en.w : 0u;
+            en = __ldg(ent + min(q + 32 + lane, tc - 1));
           }
           w = ee.x & 0xff;
           const int wmax = (int)__reduce_max_sync(FULL, (unsigned)w);
           const SYN s = ent_syndrome<SYN>(ee, w, wmax, sc.hr(), mass) ^ h.s0;
           hm = __ballot_sync(FULL, lane < lim && s == 0);
-          if (hm == 0) {  // lanes past lim hold an empty entry
-            wacc += w;
-            df_acc(tmass, mass);
-            q += lim;
+          if (hm != 0) {
+            hl = take();
+            if (hl >= 0) goto left;
           }
-        }
-        if (hm == 0) continue;
-      }
-      // the chunk's next hit
-      hl = __ffs(hm) - 1;
-      hm &= hm - 1;
-      if (lane == nhit) hq = q + hl;
-      nhit++;
-      fin = nhit >= P.L;
-      if (MODE == MODE_THR || fin) break;
-      hl = -1;
-      if (hm == 0) {
-        wacc += w;
-        df_acc(tmass, mass);
-        q += lim;
+          queried();  // lanes past lim hold an empty entry
+        } while (q < qlim);
       }
     }
+  left:
 #ifdef SG_PHASE_PROFILE
     if (t2 == 0) t2 = clock64();
 #endif
+    // the list is complete, or the order or the cap ended
+    const bool fin = nhit >= P.L || zone >= 3;
     record_list<NPL, SYN>(sc, ent, hq, listed, nhit, lane);
     listed = nhit;
     // the queries made up to here: qn, their mass `part`
@@ -1421,11 +1461,7 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
       q = qn;
       break;
     }
-    if (hm == 0) {  // that was the chunk's last hit
-      wacc += w;
-      df_acc(tmass, mass);
-      q += lim;
-    }
+    if (hm == 0) queried();  // that was the chunk's last hit
   }
 #ifdef SG_PHASE_PROFILE
   if (lane == 0) SG_PROF(5, (q + 31) / 32);
