@@ -116,11 +116,15 @@ __device__ __forceinline__ DF df_mul_f(DF a, float b) {
   const float p = __fmul_rn(a.h, b);
   return df_norm(p, fmaf(a.l, b, fmaf(a.h, b, -p)));
 }
-// running sum of nonnegative terms: the low part collects the exact rounding errors
+// running sum of nonnegative terms: the low part collects the exact rounding
+// errors (the larger high part first: Dekker's fast two-sum, the same exact
+// error as Knuth's)
 __device__ __forceinline__ void df_acc(DF &a, DF x) {
-  const DF s = df_two_sum(a.h, x.h);
-  a.h = s.h;
-  a.l = __fadd_rn(a.l, __fadd_rn(s.l, x.l));
+  const float hi = fmaxf(a.h, x.h), lo = fminf(a.h, x.h);
+  const float s = __fadd_rn(hi, lo);
+  const float err = __fsub_rn(lo, __fsub_rn(s, hi));
+  a.h = s;
+  a.l = __fadd_rn(a.l, __fadd_rn(err, x.l));
 }
 // The warp butterflies that run once per word are loops, not unrolled: the
 // kernel's per-word path is long and instruction fetch is its first stall, so
@@ -1266,6 +1270,7 @@ __device__ __forceinline__ void build_prefixes(const Scratch<NPL, SYN> &sc, SYN 
 template <int NPL, class SYN, int MODE, class Emit>
 __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams &P, const Scratch<NPL, SYN> &sc,
                                           const float (&lam)[NPL], int lane, WordResult &res, Emit emit) {
+  using LY = Layout<NPL, SYN>;
   constexpr int NM = (32 * NPL + 63) / 64;
   const int n = code.n;
 #ifdef SG_PHASE_PROFILE
@@ -1371,43 +1376,71 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
           }
         }
       } else if (MODE != MODE_LANES && sizeof(SYN) == 4 && zone < 2) {
-        // full chunks in the two- or three-rank form: one loop for both, so
-        // that its instructions are fetched once
-        const bool three = zone != 0;
-#pragma unroll 1
-        do {
-          const unsigned cur = e.x;
-          e.x = e.y;
-          e.y = e.z;
-          e.z = e.w;
-          if ((q & 96) == 96) {  // the group's last chunk
-            e = en;
-            en = __ldg(e4 + (q >> 2) + 40);  // q / 4 is 24 past the group; the table is padded by two groups
-          }
-          const uint4 r = sc.prec()[cur & 0xff];
-          const RankRec<SYN> ra = sc.hr()[(cur >> 8) & 0xff], rb = sc.hr()[(cur >> 16) & 0xff];
-          unsigned s = r.x ^ (unsigned)ra.h ^ (unsigned)rb.h;
-          w = (int)r.w;
+        // full chunks: the record of the entry's prefix, then its last ranks
+        const unsigned prec = sc.base + LY::o_pf, hr = sc.base + LY::o_hr;
+        unsigned s = 0;
+        const auto rank = [&](unsigned byte) {
+          const RankRec<SYN> v = *sptr<const RankRec<SYN>>(hr + 8 * byte);
+          s ^= (unsigned)v.h;
+          const float p = __fmul_rn(mass.h, v.t);
+          mass.l = fmaf(mass.l, v.t, fmaf(mass.h, v.t, -p));
+          mass.h = p;
+        };
+        const auto prefix = [&](unsigned cur) {
+          const uint4 r = *sptr<const uint4>(prec + 16 * __byte_perm(cur, 0u, 0x4440));
+          s = r.x;
           mass = DF{__uint_as_float(r.y), __uint_as_float(r.z)};
-          const auto mul = [&](float t) {
-            const float p = __fmul_rn(mass.h, t);
-            mass.l = fmaf(mass.l, t, fmaf(mass.h, t, -p));
-            mass.h = p;
-          };
-          mul(ra.t);
-          mul(rb.t);
-          if (three) {
-            const RankRec<SYN> rc = sc.hr()[cur >> 24];
-            s ^= (unsigned)rc.h;
-            mul(rc.t);
-          }
-          hm = __ballot_sync(FULL, s == 0);
-          if (hm != 0) {
-            hl = take();
-            if (hl >= 0) goto left;
-          }
-          queried();
-        } while (q < qe);
+          w = (int)r.w;
+          rank(__byte_perm(cur, 0u, 0x4441));
+          rank(__byte_perm(cur, 0u, 0x4442));
+        };
+        const auto advance = [&]() {  // the next group of entries
+          e = en;
+          en = __ldg(e4 + (q >> 2) + 64 - ((q >> 2) & 31));
+        };
+        // a loop for each form (a predicated third rank would cost the two-rank
+        // form its instructions); two chunks a trip in the first, which most
+        // words never leave (MODE_THR, which resumes at any chunk, takes one)
+        if (MODE == MODE_TABLE && zone == 0) {
+#pragma unroll 1
+          do {
+            const unsigned c1 = e.y;
+            prefix(e.x);
+            hm = __ballot_sync(FULL, s == 0);
+            if (hm != 0) {
+              hl = take();
+              if (hl >= 0) goto left;
+            }
+            queried();
+            prefix(c1);
+            e.x = e.z;
+            e.y = e.w;
+            if ((q & 64) != 0) advance();
+            hm = __ballot_sync(FULL, s == 0);
+            if (hm != 0) {
+              hl = take();
+              if (hl >= 0) goto left;
+            }
+            queried();
+          } while (q < qe);
+        } else {
+#pragma unroll 1
+          do {
+            const unsigned cur = e.x;
+            e.x = e.y;
+            e.y = e.z;
+            e.z = e.w;
+            if ((q & 96) == 96) advance();
+            prefix(cur);
+            if (MODE == MODE_TABLE || zone != 0) rank(cur >> 24);
+            hm = __ballot_sync(FULL, s == 0);
+            if (hm != 0) {
+              hl = take();
+              if (hl >= 0) goto left;
+            }
+            queried();
+          } while (q < qe);
+        }
       } else {
         // rank by rank, the entries read a chunk ahead
 #pragma unroll 1
