@@ -837,7 +837,7 @@ size_t persistent_scratch_bytes(int64_t F, int nr, int nc, int nm, int max_iter)
   return al256((size_t)F * nr * nc * sizeof(float)) + al256((size_t)F * std::max(nr, nc) * nm * sizeof(uint64_t)) +
          5 * al256(b_i32) +
          al256((size_t)F * 2 * max_iter * sizeof(int32_t)) + 2 * al256(b_i64) + al256((size_t)F) +
-         al256(8 * sizeof(int32_t));
+         al256(sg::CTRL_WORDS * sizeof(int32_t));
 }
 
 // The global remaining-mass region of a persistent launch: one slice per
@@ -886,7 +886,7 @@ cudaError_t persistent_enqueue(sogrand_code *c, const sogrand_code *cc, int64_t 
   int64_t *q_s = (int64_t *)take(b_i64);
   int64_t *pq_s = (int64_t *)take(b_i64);
   uint8_t *st_s = (uint8_t *)take((size_t)F);
-  a.ctrl = (int32_t *)take(8 * sizeof(int32_t));
+  a.ctrl = (int32_t *)take(sg::CTRL_WORDS * sizeof(int32_t));
   a.bits = bits;
   a.half_iters = half_iters ? half_iters : hi_s;
   a.queries = queries ? queries : q_s;
@@ -900,7 +900,7 @@ cudaError_t persistent_enqueue(sogrand_code *c, const sogrand_code *cc, int64_t 
   a.dp_blocks = sgi::sm_count_of_device() * sg::MAX_BLOCKS_PER_SM;
   a.xf_count = xf;
   a.wsum = wsum;
-  *err_dev = a.ctrl + 3;
+  *err_dev = a.ctrl + sg::CTRL_ERROR;
   sg::DevCode d = dev_code(c), dcol = dev_code(cc);
   const bool gen = cc != c || a.diag || a.nr != a.nc;  // not the square product of one code
   cudaError_t e = cudaSuccess;

@@ -193,6 +193,10 @@ __device__ __forceinline__ void tally_flush(const unsigned long long *slot, unsi
 // registers that held it are free while the search runs.
 struct WordCtx {
   int32_t f, li, wd, rows;
+  // persistent form: the queries and the largest query count of the words
+  // decoded since the frame's counters were last brought up to date
+  int32_t qmax, words;
+  int64_t queries;
 };
 static_assert(sizeof(WordCtx) <= 32, "the word's lambda follows the context in the frame-check area");
 
@@ -262,13 +266,19 @@ __device__ __forceinline__ int product_word(const DevCode &code, const SisoParam
     if (NPL & 1) reinterpret_cast<unsigned *>(a.hb + at * NM)[NPL] = 0u;  // the upper half of the last u64
     if (a.wq) a.wq[at] = res.queries;
     if (res.queries >= 0) {
-      atomicAdd(reinterpret_cast<unsigned long long *>(a.queries + f), (unsigned long long)res.queries);
-      atomicMax(a.hmax + f, res.queries);
+      if constexpr (COHERENT) {
+        WordCtx *c = reinterpret_cast<WordCtx *>(sc.W());
+        c->queries += res.queries;
+        c->qmax = max(c->qmax, res.queries);
+      } else {
+        atomicAdd(reinterpret_cast<unsigned long long *>(a.queries + f), (unsigned long long)res.queries);
+        atomicMax(a.hmax + f, res.queries);
+      }
       sc.tally()[0] += (unsigned long long)res.wsum;
     }
     if (res.flags) {
       sc.tally()[1] += res.flags & 1;
-      if ((res.flags & 2) && a.ctrl) atomicExch(a.ctrl + 3, 2);  // stops a persistent launch: reported as a timeout
+      if ((res.flags & 2) && a.ctrl) atomicExch(a.ctrl + CTRL_ERROR, 2);  // stops a persistent launch: reported as a timeout
     }
   }
   __syncwarp();
@@ -539,18 +549,13 @@ __device__ __forceinline__ int32_t slot_value(int li, int half) {
   return (half & 1) ? v : -v;
 }
 
-// Draw a word ticket and wait until its slot of the frame-half list is filled.
-// Returns the signed slot value, or 0 when the list is done (every frame
-// finished or parked) or the launch's error word a.ctrl[3] is set.  The wait
-// backs off exponentially and gives up after max_spin microseconds of sleep,
-// setting the error word.  All reads of shared state are made by lane 0 and
-// broadcast, so the whole warp takes the same branch.
-__device__ __forceinline__ int sched_take(const ProductArgs &a, int slot_n, int lane, int *word_out, int *waited) {
-  int ticket = 0;
-  if (lane == 0) ticket = atomicAdd(a.ctrl + 1, 1);
-  ticket = __shfl_sync(FULL, ticket, 0);
-  const int slot = ticket / slot_n;
-  *word_out = ticket - slot * slot_n;
+// Wait until slot `slot` of the frame-half list is filled.  Returns its signed
+// value, or 0 when the list is done (every frame finished or parked) or the
+// launch's error word is set.  The wait backs off exponentially and gives up
+// after max_spin microseconds of sleep, setting the error word.  All reads of
+// shared state are made by lane 0 and broadcast, so the whole warp takes the
+// same branch.
+__device__ __forceinline__ int sched_wait(const ProductArgs &a, int slot, int lane, int *waited) {
   const bool real = slot < a.n_frames * a.max_half;  // a frame has at most max_half halves
   int v = 0;
   unsigned slept = 0, nap = 64;  // slept: microseconds / 1.024
@@ -560,10 +565,10 @@ __device__ __forceinline__ int sched_take(const ProductArgs &a, int slot_n, int 
       if (real) v = ld_acquire_gpu(a.queue + slot);
       // an error, or every frame finished and this ticket has no work
       const volatile int32_t *ctrl = a.ctrl;
-      if (ctrl[3] != 0)
+      if (ctrl[CTRL_ERROR] != 0)
         stop = 1;
       else if (v == 0)
-        stop = ctrl[2] >= a.n_frames;
+        stop = ctrl[CTRL_DONE] >= a.n_frames;
     }
     stop = __shfl_sync(FULL, stop, 0);
     v = __shfl_sync(FULL, v, 0);
@@ -571,7 +576,7 @@ __device__ __forceinline__ int sched_take(const ProductArgs &a, int slot_n, int 
     if (v != 0) break;
     *waited = 1;
     if ((slept >> 10) > (unsigned)a.max_spin) {
-      if (lane == 0) atomicExch(a.ctrl + 3, 1);
+      if (lane == 0) atomicExch(a.ctrl + CTRL_ERROR, 1);
       return 0;
     }
     __nanosleep(nap);
@@ -608,14 +613,14 @@ __device__ __forceinline__ void frame_after_half(const DevCode &wc, const DevCod
   }
   if (bad || ok || half >= a.max_half) {
     frame_finish<NPL>(a, f, rows, half, bad ? 2 : (ok ? 0 : 1), W, lane);
-    if (lane == 0) atomicAdd(a.ctrl + 2, 1);
+    if (lane == 0) atomicAdd(a.ctrl + CTRL_DONE, 1);
   } else if (lane == 0) {
     a.half_cur[f] = half + 1;
     a.done_words[f] = 0;
     if (half >= stop) {  // parked: resumes at half + 1 in a later launch
-      atomicAdd(a.ctrl + 2, 1);
+      atomicAdd(a.ctrl + CTRL_DONE, 1);
     } else {
-      const int t = atomicAdd(a.ctrl + 0, 1);  // < nslots: every frame appends at most max_half - 1 times
+      const int t = atomicAdd(a.ctrl + CTRL_SLOTS, 1);  // < nslots: every frame appends at most max_half - 1 times
       st_release_gpu(a.queue + t, slot_value(li, half + 1));
     }
   }
@@ -648,53 +653,86 @@ __global__ void __launch_bounds__(TPB, resident_blocks(MINB))
   bind_scratch(sc, smem, warp, LY::warp_bytes, block_dp_area(smem, LY::warp_bytes, a.dp_area, a.dp_stride), tl);
   const int slot_n = GEN ? max(a.nr, a.nc) : rowc.n;  // tickets per list slot: the most words in a half
   tally_clear(sc.tally(), lane);
-  if (lane == 0) atomicAdd(a.ctrl + 4, 1);  // one more active warp
+  if (lane == 0) atomicAdd(a.ctrl + CTRL_WARPS, 1);  // one more active warp
   int waited = 0;
+  int ticket = 0, left = 0;  // the next ticket and how many more of its run are this warp's
+  int slot = -1, v = 0;      // the slot last waited for and its value
+  WordCtx *ctx = reinterpret_cast<WordCtx *>(sc.W());
   for (;;) {
-    // Drain: a warp leaves once the unfinished frames cannot use it (each has
-    // at most slot_n words in flight), so the SMs go to other work sharing
-    // the GPU (the parallel kernels of the mixed form); the warps that stay
-    // can always take every word that becomes available.  Decided before a
-    // ticket is drawn (a drawn ticket is always decoded), and only once the
-    // warp has had to wait for work: while the list runs ahead of the
-    // tickets the check is skipped.
-    int leave = 0;
-    if (waited && lane == 0) {
-      const int64_t need = (a.n_frames - (int64_t)__ldcg(a.ctrl + 2)) * slot_n;
-      if ((int64_t)__ldcg(a.ctrl + 4) - 1 >= need) {
-        if ((int64_t)atomicSub(a.ctrl + 4, 1) - 1 >= need)
-          leave = 1;
-        else
-          atomicAdd(a.ctrl + 4, 1);
+    if (left == 0) {
+      // Drain: a warp leaves once the unfinished frames cannot use it (each has
+      // at most slot_n words in flight), so the SMs go to other work sharing
+      // the GPU (the parallel kernels of the mixed form); the warps that stay
+      // can always take every word that becomes available.  Decided before a
+      // ticket is drawn (a drawn ticket is always decoded), and only once the
+      // warp has had to wait for work: while the list runs ahead of the
+      // tickets the check is skipped.
+      int leave = 0;
+      if (waited && lane == 0) {
+        const int64_t need = (a.n_frames - (int64_t)__ldcg(a.ctrl + CTRL_DONE)) * slot_n;
+        if ((int64_t)__ldcg(a.ctrl + CTRL_WARPS) - 1 >= need) {
+          if ((int64_t)atomicSub(a.ctrl + CTRL_WARPS, 1) - 1 >= need)
+            leave = 1;
+          else
+            atomicAdd(a.ctrl + CTRL_WARPS, 1);
+        }
       }
+      if (__shfl_sync(FULL, leave, 0)) {
+        // this block has begun to leave: a decoder launched as a programmatic
+        // dependent of this one may start (no effect otherwise)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        break;
+      }
+      left = waited ? 1 : a.run;
+      if (lane == 0) ticket = atomicAdd(a.ctrl + CTRL_TICKETS, left);
+      ticket = __shfl_sync(FULL, ticket, 0);
     }
-    if (__shfl_sync(FULL, leave, 0)) {
-      // this block has begun to leave: a decoder launched as a programmatic
-      // dependent of this one may start (no effect otherwise)
-      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-      break;
+    const int at = ticket / slot_n, w = ticket - at * slot_n;
+    ticket++;
+    left--;
+    if (at != slot) {
+      slot = at;
+      v = sched_wait(a, slot, lane, &waited);
+      if (v == 0) break;
+      if (lane == 0) {
+        ctx->qmax = ctx->words = 0;
+        ctx->queries = 0;
+      }
+      __syncwarp();
     }
-    int w;
-    const int v = sched_take(a, slot_n, lane, &w, &waited);
-    if (v == 0) break;
     const bool rows = v > 0;  // the slot's half is odd: a row half
-    const int li = ((rows ? v : -v) >> 1) - 1;  // list index
     const DevCode &code = GEN ? (rows ? rowc : colc) : rowc, &xcode = GEN ? (rows ? colc : rowc) : rowc;
     const int n = xcode.n;  // words in this half
-    // a ticket past this half's words (codes of different lengths); decided
-    // from the slot, since the frame may already be in its next half
-    if (GEN && w >= n) continue;
-    int f = a.frame_list ? a.frame_list[li] : li;
-    const int q = product_word<NPL, SYN, true, GEN, MODE>(code, P, a, sc, f, li, w, rows, rows && (v & 1), lane);
-    f = *reinterpret_cast<const volatile int *>(sc.W());
-    if (lane == 0 && q < 0) atomicExch(a.bad + f, 1);
-    __syncwarp();  // every lane's L_E and hard decision, then lane 0 releases them
-    int done = 0;
-    if (lane == 0) done = atom_add_acq_rel_gpu(a.done_words + f, 1);  // acquire: the frame's other words
-    done = __shfl_sync(FULL, done, 0);
-    if (done != n - 1) continue;
-    const int li2 = *(reinterpret_cast<const volatile int *>(sc.W()) + 1);
-    frame_after_half<NPL, GEN>(code, xcode, a, f, li2, sc.base + LY::o_w, lane);
+    // (a ticket past this half's words, of codes of different lengths, has no
+    // word; decided from the slot, since the frame may already be in its next half)
+    if (!GEN || w < n) {
+      const int li = ((rows ? v : -v) >> 1) - 1;  // list index
+      const int f = a.frame_list ? a.frame_list[li] : li;
+      const int q = product_word<NPL, SYN, true, GEN, MODE>(code, P, a, sc, f, li, w, rows, rows && (v & 1), lane);
+      if (lane == 0) {
+        ctx->words++;
+        if (q < 0) atomicExch(a.bad + ctx->f, 1);
+      }
+      __syncwarp();  // every lane's L_E and hard decision, then lane 0 releases them
+      // the frame's counters once for the words of it that were drawn together
+      if (left == 0 || w == n - 1) {
+        int last = 0;
+        if (lane == 0) {
+          const int fr = ctx->f, words = ctx->words;
+          atomicAdd(reinterpret_cast<unsigned long long *>(a.queries + fr), (unsigned long long)ctx->queries);
+          atomicMax(a.hmax + fr, ctx->qmax);
+          last = atom_add_acq_rel_gpu(a.done_words + fr, words) + words == n;  // acquire: the frame's other words
+          ctx->qmax = ctx->words = 0;
+          ctx->queries = 0;
+        }
+        if (__shfl_sync(FULL, last, 0)) {
+          const volatile WordCtx *vc = ctx;
+          const int fr = vc->f, fl = vc->li;
+          frame_after_half<NPL, GEN>(code, xcode, a, fr, fl, sc.base + LY::o_w, lane);
+          slot = -1;  // the frame check has used the words' context
+        }
+      }
+    }
   }
   tally_flush(sc.tally(), a.wsum, a.xf_count, lane);
 }
@@ -729,11 +767,11 @@ static __global__ void k_persistent_init(const ProductArgs a) {
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    a.ctrl[0] = (int32_t)F;  // next slot to reserve
-    a.ctrl[1] = 0;           // word tickets drawn
-    a.ctrl[2] = 0;           // frames finished
-    a.ctrl[3] = 0;           // error
-    a.ctrl[4] = 0;           // active warps
+    a.ctrl[CTRL_SLOTS] = (int32_t)F;  // next slot to reserve
+    a.ctrl[CTRL_TICKETS] = 0;           // word tickets drawn
+    a.ctrl[CTRL_DONE] = 0;           // frames finished
+    a.ctrl[CTRL_ERROR] = 0;           // error
+    a.ctrl[CTRL_WARPS] = 0;           // active warps
   }
 }
 
@@ -837,7 +875,8 @@ cudaError_t launch_product_init(const DevCode &code, const ProductArgs &a, cudaS
 
 template <int NPL, class SYN, bool GEN>
 cudaError_t launch_product_persistent(const DevCode &rowc, const DevCode &colc, const SisoParams &P,
-                                      const ProductArgs &a, cudaStream_t s, int part) {
+                                      const ProductArgs &a_, cudaStream_t s, int part) {
+  ProductArgs a = a_;
   if (a.n_frames <= 0) return cudaSuccess;
   cudaError_t e = cudaSuccess;
   if (part == PERSISTENT_ALL || part == PERSISTENT_INIT) {
@@ -866,6 +905,15 @@ cudaError_t launch_product_persistent(const DevCode &rowc, const DevCode &colc, 
   if (a.grid_cap > 0 && a.grid_cap < cap) cap = a.grid_cap;
   if (a.dp_area && a.dp_blocks < cap) cap = a.dp_blocks;  // one slice of the region per block
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(cap, want));
+  // Tickets drawn at once: up to 8 while every warp has at least 8 such runs
+  // in the first half alone, else fewer, so that a small batch spreads over
+  // all warps.  A run saves the draw, the look at the list and the release of
+  // the finished words for all but one of its words: with one ticket a draw
+  // the ticket counter's L2 line took three accesses a word and bound the
+  // launch (eBCH(64,57)^2, 20,000 frames: 26.7 ms at runs of 1, 23.1 at 2,
+  // 22.1 at 4, 21.6 at 8).
+  const int64_t per_warp = words / ((int64_t)grid * WARPS_PER_BLOCK);
+  a.run = per_warp >= 64 ? 8 : (per_warp >= 32 ? 4 : (per_warp >= 16 ? 2 : 1));
   if (part == PERSISTENT_DECODE_PDL) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);

@@ -53,7 +53,8 @@ struct ProductArgs {
   int32_t *half_cur;          // [F] current half iteration of each frame
   int32_t *done_words;        // [F] words of the current half completed
   int32_t *bad;               // [F] a non-finite input was seen
-  int32_t *ctrl;              // [8] slots reserved, word tickets, finished frames, error, active warps
+  int32_t *ctrl;              // [CTRL_WORDS] the scheduler's words, indexed by CTRL_*
+  int32_t run;                // word tickets a warp draws at once while the list runs ahead of it
   int32_t max_spin;           // microseconds of accumulated back-off without work before giving up
   int32_t *half_stop;         // [F] or null: park the frame after this half (serving epochs)
   // serving: the launch decodes the frames named by a list (buffer indices;
@@ -70,6 +71,17 @@ struct ProductArgs {
   // shared memory
   unsigned char *dp_area;
   int32_t dp_stride, dp_blocks;
+};
+
+// The scheduler's words, each in a 128-byte line of its own: every warp draws
+// tickets from one of them, and its L2 line takes no other traffic.
+enum : int {
+  CTRL_SLOTS = 0,      // list slots reserved
+  CTRL_TICKETS = 32,   // word tickets drawn
+  CTRL_DONE = 64,      // frames finished or parked
+  CTRL_ERROR = 96,     // 1: a wait gave up, 2: a remaining-mass lock was not taken
+  CTRL_WARPS = 128,    // active warps
+  CTRL_WORDS = 160
 };
 
 template <int NPL, class SYN>

@@ -85,7 +85,7 @@ struct Pool {
   int64_t *queries = nullptr, *par_queries = nullptr;
   int32_t *h_list = nullptr;   // pinned [slots]
   uint8_t *h_status = nullptr; // pinned [slots]
-  int32_t *h_ctrl = nullptr;   // pinned [4]
+  int32_t *h_ctrl = nullptr;   // pinned [1]: the launch's error word
   cudaStream_t stream = nullptr;
   std::map<int32_t, int32_t> free_runs;  // free slot ranges: first -> length (coalesced)
   int64_t free_count = 0;
@@ -177,7 +177,7 @@ size_t carve(Pool &p, int max_iter, char *mem) {
   p.queries = (int64_t *)take(S * 8);
   p.par_queries = (int64_t *)take(S * 8);
   p.queue = (int32_t *)take(S * 2 * max_iter * 4);
-  p.ctrl = (int32_t *)take(32);
+  p.ctrl = (int32_t *)take(sg::CTRL_WORDS * sizeof(int32_t));
   p.dp_area = (unsigned char *)take((size_t)p.dp_blocks * p.dp_stride);
   return off;
 }
@@ -220,7 +220,7 @@ void retire(sogrand_server *sv, Pool &p) {
   std::vector<int32_t> still;
   std::vector<Request *> completed;
   still.reserve(p.active.size());
-  const bool failed = p.h_ctrl[3] != 0;
+  const bool failed = p.h_ctrl[0] != 0;
   for (int32_t e : p.active) {
     const int32_t slot = e < 0 ? -e - 1 : e;
     if (!failed && p.h_status[slot] == 255) {
@@ -331,7 +331,7 @@ cudaError_t launch(sogrand_server *sv, Pool &p, int64_t total_words) {
   const sg::SisoParams P = sgi::siso_params_of(sv->L, sv->cap, sv->thr);
   if (e == cudaSuccess) e = sgi::launch_persistent_for(p.code, P, a, p.stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(p.h_status, p.status, p.slots, cudaMemcpyDeviceToHost, p.stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(p.h_ctrl, p.ctrl, 16, cudaMemcpyDeviceToHost, p.stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(p.h_ctrl, p.ctrl + sg::CTRL_ERROR, 4, cudaMemcpyDeviceToHost, p.stream);
   p.launched_words = words;
   return e;
 }
