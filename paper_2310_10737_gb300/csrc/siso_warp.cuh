@@ -1209,6 +1209,13 @@ __device__ __forceinline__ void record_list(const Scratch<NPL, SYN> &sc, const u
 // (ent_syndrome).  64-bit syndromes leave no room for the record in 16 bytes
 // and always take the last form.
 
+struct FalseTag {
+  static constexpr bool value = false;
+};
+struct TrueTag {
+  static constexpr bool value = true;
+};
+
 // Where the query loop takes its patterns and when it stops.
 enum : int {
   MODE_TABLE = 0,  // the order tables, no threshold rule
@@ -1376,70 +1383,72 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
           }
         }
       } else if (MODE != MODE_LANES && sizeof(SYN) == 4 && zone < 2) {
-        // full chunks: the record of the entry's prefix, then its last ranks
+        // full chunks, two at a time: the record of each entry's prefix, then
+        // its last ranks.  Both chunks are tested before either is taken, so
+        // a warp alone on its SM waits for one chunk's loads and products, not
+        // two.  (MODE_THR can resume at a pair's second chunk.)
         const unsigned prec = sc.base + LY::o_pf, hr = sc.base + LY::o_hr;
-        unsigned s = 0;
-        const auto rank = [&](unsigned byte) {
-          const RankRec<SYN> v = *sptr<const RankRec<SYN>>(hr + 8 * byte);
-          s ^= (unsigned)v.h;
-          const float p = __fmul_rn(mass.h, v.t);
-          mass.l = fmaf(mass.l, v.t, fmaf(mass.h, v.t, -p));
-          mass.h = p;
-        };
-        const auto prefix = [&](unsigned cur) {
+        const auto test = [&](unsigned cur, auto three, DF &m, int &wt) {
           const uint4 r = *sptr<const uint4>(prec + 16 * __byte_perm(cur, 0u, 0x4440));
-          s = r.x;
-          mass = DF{__uint_as_float(r.y), __uint_as_float(r.z)};
-          w = (int)r.w;
+          unsigned s = r.x;
+          m = DF{__uint_as_float(r.y), __uint_as_float(r.z)};
+          wt = (int)r.w;
+          const auto rank = [&](unsigned byte) {
+            const RankRec<SYN> v = *sptr<const RankRec<SYN>>(hr + 8 * byte);
+            s ^= (unsigned)v.h;
+            const float p = __fmul_rn(m.h, v.t);
+            m.l = fmaf(m.l, v.t, fmaf(m.h, v.t, -p));
+            m.h = p;
+          };
           rank(__byte_perm(cur, 0u, 0x4441));
           rank(__byte_perm(cur, 0u, 0x4442));
+          if constexpr (decltype(three)::value) rank(cur >> 24);
+          return s;
         };
-        const auto advance = [&]() {  // the next group of entries
-          e = en;
-          en = __ldg(e4 + (q >> 2) + 64 - ((q >> 2) & 31));
-        };
-        // a loop for each form (a predicated third rank would cost the two-rank
-        // form its instructions); two chunks a trip in the first, which most
-        // words never leave (MODE_THR, which resumes at any chunk, takes one)
-        if (MODE == MODE_TABLE && zone == 0) {
+        const auto pairs = [&](auto three) {  // whether the search leaves
 #pragma unroll 1
           do {
-            const unsigned c1 = e.y;
-            prefix(e.x);
-            hm = __ballot_sync(FULL, s == 0);
-            if (hm != 0) {
-              hl = take();
-              if (hl >= 0) goto left;
+            DF ma, mb;
+            int wa, wb;
+            const unsigned sa = test(e.x, three, ma, wa), sb = test(e.y, three, mb, wb);
+            const unsigned ha = __ballot_sync(FULL, sa == 0), hb = __ballot_sync(FULL, sb == 0);
+            if (MODE != MODE_THR || (q & 32) == 0) {
+              if (ha != 0) {
+                hm = ha;
+                mass = ma;
+                w = wa;
+                hl = take();
+                if (hl >= 0) return true;
+              }
+              wacc += wa;
+              df_acc(tmass, ma);
+              q += 32;
             }
-            queried();
-            prefix(c1);
             e.x = e.z;
             e.y = e.w;
-            if ((q & 64) != 0) advance();
-            hm = __ballot_sync(FULL, s == 0);
-            if (hm != 0) {
-              hl = take();
-              if (hl >= 0) goto left;
+            if ((q & 64) != 0) {  // the next group of entries
+              e = en;
+              en = __ldg(e4 + (q >> 2) + 64 - ((q >> 2) & 31));
             }
-            queried();
+            if (hb != 0) {
+              hm = hb;
+              mass = mb;
+              w = wb;
+              hl = take();
+              if (hl >= 0) return true;
+            }
+            wacc += wb;
+            df_acc(tmass, mb);
+            q += 32;
           } while (q < qe);
+          return false;
+        };
+        // a loop for each form: a predicated third rank would cost the
+        // two-rank form its instructions
+        if (zone == 0) {
+          if (pairs(FalseTag{})) goto left;
         } else {
-#pragma unroll 1
-          do {
-            const unsigned cur = e.x;
-            e.x = e.y;
-            e.y = e.z;
-            e.z = e.w;
-            if ((q & 96) == 96) advance();
-            prefix(cur);
-            if (MODE == MODE_TABLE || zone != 0) rank(cur >> 24);
-            hm = __ballot_sync(FULL, s == 0);
-            if (hm != 0) {
-              hl = take();
-              if (hl >= 0) goto left;
-            }
-            queried();
-          } while (q < qe);
+          if (pairs(TrueTag{})) goto left;
         }
       } else {
         // rank by rank, the entries read a chunk ahead
