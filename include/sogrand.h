@@ -263,11 +263,11 @@ int gldpc_decode(sogrand_code *code, int64_t n_frames, const float *llr_ch, int 
                  product_decode_stats *stats, void *stream);
 
 /*
- * Schedule of a code's decoding kernels: the number of resident blocks per SM
- * (128 threads each) they are compiled for, 8 (64 registers a thread) or 12
- * (40 registers).  Which is faster depends on the code (register pressure of
- * its syndrome width and list against the latency the extra warps hide) and
- * is measured by sogrand_code_tune.  The default until tuned: 12 for
+ * Schedule of a code's decoding kernels: 8 (compiled for 8 resident blocks of
+ * 128 threads per SM, 64 registers a thread) or 12 (the schedule of more
+ * warps: 48 registers a thread, 10 resident blocks).  Which is faster depends
+ * on the code (register pressure of its syndrome width and list against the
+ * latency the extra warps hide) and is measured by sogrand_code_tune.  The default until tuned: 12 for
  * n <= 64, else 8.
  *   minb     0 (query only), 8 or 12
  *   current  HOST out (may be NULL): the schedule in force
@@ -293,8 +293,9 @@ int sogrand_code_dp_area(sogrand_code *code, int where, int *current);
  * increasing cost = sum of reliability ranks + c * Hamming weight, the
  * patterns of one cost and weight being the partitions of that rank sum into
  * distinct parts <= n):
- *   0  read from the code's precomputed order table (one 16-byte entry per
- *      query, copied ahead into shared memory; the default, and the faster);
+ *   0  read from the code's precomputed order table (the head of every order
+ *      in 4-byte entries, past it one 16-byte entry per query; the default,
+ *      and the faster);
  *   1  enumerated by the lanes themselves: lane j of a chunk of 32 queries
  *      finds the (cost, weight) group of its query from the order's group
  *      list and unranks its partition with a table of subset counts.
@@ -302,7 +303,7 @@ int sogrand_code_dp_area(sogrand_code *code, int where, int *current);
  * to sogrand_decode and to the batched form of square product codes
  * (product_decode_persistent, product_decode_mixed, product_decode_host, the
  * server) when thr = 0; every other case reads the table, and the
- * remaining-mass computation reads it either way.  Source 1 runs kernels of
+ * listed words and the remaining-mass computation read it either way.  Source 1 runs kernels of
  * their own, so the table path's kernels are unaffected by it.
  *   source   -1 (query only), 0 or 1
  *   current  HOST out (may be NULL): the source in force
@@ -313,11 +314,11 @@ int sogrand_code_order_source(sogrand_code *code, int source, int *current);
 /*
  * Autotuner: decodes a sample of frames (device [n_frames][n][n] LLRs, with
  * the decode parameters of the intended workload) with the batched form
- * under each schedule (8 or 12 blocks per SM, each with the remaining-mass
+ * under each schedule (8 or 12, each with the remaining-mass
  * area in shared and in global memory), twice each (the first run warms
  * caches), and keeps the fastest for this code.  Synchronous on `stream`;
  * writes no caller buffer but `chosen` (HOST, may be NULL: 8 or 12) and ms_out
- * (HOST [2] or NULL: the better timed run for 8 and for 12 blocks per SM); the
+ * (HOST [2] or NULL: the better timed run for schedule 8 and for 12); the
  * chosen placement is read with sogrand_code_dp_area.  Errors: as
  * product_decode_persistent; EINVAL also for n_frames < 1.
  */

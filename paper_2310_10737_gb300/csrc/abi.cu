@@ -26,7 +26,7 @@ struct sogrand_code {
   sg::DevOrder ord{};
   sg::DevGroups grp{};
   int jmax = 1;
-  int minb = 12;  // schedule: resident blocks per SM (8 or 12), see sogrand_code_tune
+  int minb = 12;  // schedule: 8 or 12, see sogrand_code_schedule
   int dp_global = 1;  // schedule: the batched forms keep the remaining-mass area in global memory
   int ord_lanes = 0;  // 1: lanes enumerate the query order instead of reading the order table
   int64_t tab_cap = 0;
@@ -583,7 +583,7 @@ int sogrand_code_create(int n, int k, const uint8_t *H, int even, sogrand_code *
   c->even = even;
   c->c_max = n;
   c->nm = (n + 63) / 64;
-  // default schedule until tuned: 12 blocks per SM (40 registers) for codes
+  // default schedule until tuned: 12 (10 blocks per SM, 48 registers) for codes
   // of up to 64 bits, else 8 (64 registers)
   c->minb = n <= 64 ? 12 : 8;
   // and the remaining-mass area in global memory for the others (they gain L1)

@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(TPB, resident_blocks(MINB)) k_decode(const __g
       lam[k] = x;
     }
     WordResult res;
-    siso_word<NPL, SYN, MODE>(code, P, sc, lam, lane, res, [&](int k, float x, float lapp, bool listed) {
+    siso_word<NPL, SYN, MODE>(code, P, sc, lam, lane, res, [] {}, [&](int k, float x, float lapp, bool listed) {
       const int i = lane + 32 * k;
       if (i < n) {
         if (a.llr_app) a.llr_app[base + i] = lapp;
@@ -229,6 +229,11 @@ __device__ __forceinline__ int product_word(const DevCode &code, const SisoParam
 #endif
   const int n = code.n, nr = GEN ? a.nr : n, fsz = nr * (GEN ? a.nc : n);
   const bool diag = GEN && a.diag;
+  // the word's bits lie `step` positions apart for every 32 (a wrapped diagonal's do not)
+  const auto position = [&](int k, int w, bool r) {
+    if (diag) return bit_offset(lane + 32 * k, w, nr, r, diag);
+    return (r ? w * nr + lane : lane * nr + w) + k * (r ? 32 : 32 * nr);
+  };
   float lam[NPL];
   {
     const size_t fb = (size_t)f * fsz;
@@ -239,7 +244,7 @@ __device__ __forceinline__ int product_word(const DevCode &code, const SisoParam
       const int i = lane + 32 * k;
       lam[k] = ext[k] = 0.f;
       if (i < n) {
-        const int pos = bit_offset(i, wd, nr, rows, diag);
+        const int pos = position(k, wd, rows);
         lam[k] = __ldg(ch + pos);
         if (!first) ext[k] = ld_state<COHERENT>(le + pos);
       }
@@ -252,18 +257,28 @@ __device__ __forceinline__ int product_word(const DevCode &code, const SisoParam
   if (lane == 0) *reinterpret_cast<int4 *>(sc.W()) = make_int4(f, li, wd, rows);
   __syncwarp();
   const volatile WordCtx *vc = reinterpret_cast<const volatile WordCtx *>(sc.W());
-  siso_word<NPL, SYN, MODE>(code, P, sc, lam, lane, res, [&](int k, float x, float lapp, bool listed) {
-    const int i = lane + 32 * k;
-    if (i < n)
-      a.le[(size_t)vc->f * fsz + bit_offset(i, vc->wd, nr, vc->rows != 0, diag)] = listed ? __fsub_rn(lapp, x) : 0.f;
-    const unsigned hb = __ballot_sync(FULL, i < n && lapp < 0.f);
-    if (lane == 0) reinterpret_cast<unsigned *>(a.hb + ((size_t)vc->f * (GEN ? a.hbw : n) + vc->wd) * NM)[k] = hb;
-  });
-  f = vc->f;
-  wd = vc->wd;
+  // where the word's L_E and hard decision go, set once the search has ended
+  float *le = nullptr;
+  unsigned *hb = nullptr;
+  size_t at = 0;
+  siso_word<NPL, SYN, MODE>(
+      code, P, sc, lam, lane, res,
+      [&]() {
+        f = vc->f;
+        wd = vc->wd;
+        rows = vc->rows != 0;
+        le = a.le + (size_t)f * fsz;
+        at = (size_t)f * (GEN ? a.hbw : n) + wd;
+        hb = reinterpret_cast<unsigned *>(a.hb + at * NM);
+      },
+      [&](int k, float x, float lapp, bool listed) {
+        const bool in = lane + 32 * k < n;
+        if (in) le[position(k, wd, rows)] = listed ? __fsub_rn(lapp, x) : 0.f;
+        const unsigned h = __ballot_sync(FULL, in && lapp < 0.f);
+        if (lane == 0) hb[k] = h;
+      });
   if (lane == 0) {
-    const size_t at = (size_t)f * (GEN ? a.hbw : n) + wd;
-    if (NPL & 1) reinterpret_cast<unsigned *>(a.hb + at * NM)[NPL] = 0u;  // the upper half of the last u64
+    if (NPL & 1) hb[NPL] = 0u;  // the upper half of the last u64
     if (a.wq) a.wq[at] = res.queries;
     if (res.queries >= 0) {
       if constexpr (COHERENT) {
@@ -801,10 +816,10 @@ inline int grid_for(K kernel, int smem, int64_t warps_needed) {
   return (int)blocks;
 }
 
-// The schedule a launch runs: the code's, except that the 12-block kernels
-// (40 registers, more spills per word) are used only when the launch has more
-// words than the 8-block grid has warps; a smaller batch gains nothing from
-// the extra warps and decodes each word faster at 64 registers.
+// The schedule a launch runs: the code's, except that schedule 12's kernels
+// (48 registers) are used only when the launch has more words than the 8-block
+// grid has warps; a smaller batch gains nothing from the extra warps and
+// decodes each word faster at 64 registers.
 inline int launch_minb(int minb, int64_t words) {
   return (minb == 12 && words > (int64_t)sm_count() * 8 * WARPS_PER_BLOCK) ? 12 : 8;
 }

@@ -11,13 +11,13 @@
 // reliabilities quantised to 1/256.
 //
 // Warp mapping: lane l holds bits l, l+32, ... (NPL per lane).  The word's
-// |lambda| are bitonic-sorted across the warp (64-bit keys |lambda|:index so
-// ties fall to the lower index) and the H columns are permuted into rank order
+// |lambda| are bitonic-sorted across the warp (32-bit keys of |lambda| and the
+// index, so ties fall to the lower index; the exact order is restored where
+// the key's dropped bits decide) and the H columns are permuted into rank order
 // in shared memory.  The query order depends only on (n, c, parity class), so
-// it is read from a flattened table: every chunk of 32 consecutive queries is
-// one coalesced 512-byte copy (cp.async into the warp's shared slots, issued
-// while the previous chunk is tested), lane j takes query q0 + j, XORs its pattern's
-// H columns into the syndrome of y and reports a hit; __ballot_sync + __ffs
+// it is read from a flattened table, in chunks of 32 consecutive queries: lane
+// j takes query q0 + j, XORs its pattern's H columns (those of a shared prefix
+// at once) into the syndrome of y and reports a hit; __ballot_sync + __ffs
 // keep the hits in query order, so list, stop point and query count are those
 // of a sequential decoder.
 //
@@ -50,7 +50,7 @@ namespace sg {
 
 #ifdef SG_PHASE_PROFILE
 // [0] prologue cycles [1] query-loop cycles [2] remainder cycles [3] soft-output
-// cycles [4] words [5] query chunks [6] - [7] DP ranks [8] XF fallbacks [9] smem DP
+// cycles [4] words [5] query chunks [6] DP words [7] DP ranks [8] XF fallbacks
 // Every translation unit has its own copy of the counters (no relocatable
 // device code), so each registers a reader that sogrand_debug_phase sums.
 __device__ unsigned long long g_phase[16];
@@ -248,7 +248,7 @@ struct Layout {
   // (A separate area would cost 1 KB per block, which moved the shared-memory
   // carveout of the 8-block schedule up a step and shrank L1 by a quarter.)
   static constexpr int o_lam = o_w + 32;
-  static constexpr int HEAD = NPL + 4;  // words after lambda: see Scratch::headv
+  static constexpr int HEAD = NPL + 5;  // words after lambda: see Scratch::headv
   static_assert(32 + 4 * NT + 4 * HEAD <= 8 * NT * NM, "lambda and the word head fit in the frame-check area");
   // Prefix records of the query loop (uint4[FAST_SLOTS]); or, where a chunk is
   // tested from the 16-byte entries, uint4[32], the next chunk's entries.
@@ -299,7 +299,7 @@ struct Scratch {
   __device__ float *lamv() const { return sptr<float>(base + LY::o_lam); }
   __device__ float lam_at(int i) const { return *sptr<const volatile float>(base + LY::o_lam + 4 * i); }
   // after lambda: the word's hard decision words (NPL) and 1-line parameter,
-  // then (threshold rule) whether the double-float class total is known and it
+  // then (threshold rule) which class totals are known, and they
   __device__ unsigned *headv() const { return sptr<unsigned>(base + LY::o_lam + 4 * LY::NT); }
   __device__ unsigned head_at(int k) const { return *sptr<const volatile unsigned>(base + LY::o_lam + 4 * LY::NT + 4 * k); }
   __device__ unsigned char *tail() const { return dp; }
@@ -808,49 +808,63 @@ __device__ __forceinline__ Remaining remaining_log2_dp(const Scratch<NPL, SYN> &
 // the operands (FP32 rounding of about 4e-6 of them moves it by at most 2e-4
 // relative), in double-float when it is at least 2^-26 of them (rounding of a
 // few 2^-46 moves it by at most about 1e-5 relative).  Otherwise the
-// unqueried patterns are summed directly.  KEEP: the double-float class total
-// is kept with the word's head (the threshold rule asks at every listed word).
+// unqueried patterns are summed directly.  KEEP: the class totals are kept
+// with the word's head (the threshold rule asks at every listed word).
 template <bool KEEP, int NPL, class SYN>
 __device__ __forceinline__ Remaining remaining_log2(const Scratch<NPL, SYN> &sc, const uint4 *ent,
                                                     const uint16_t *cost, int tc, int qs, int n, int cls, int lane,
                                                     DF tq) {
   // class total of the nonzero patterns: prod_e (1 + y t_e) as (even - 1, odd)
-  float u = 0.f, b = 0.f;
+  unsigned *kept = sc.headv() + NPL + 1;  // [0] bit 0: [3] is known, bit 1: [1], [2] are
+  const unsigned known = KEEP ? __shfl_sync(FULL, sc.head_at(NPL + 1), 0) : 0u;
+  float enz;
+  if (KEEP && known != 0) {
+    enz = __uint_as_float(sc.head_at(NPL + 4));
+  } else {
+    float u = 0.f, b = 0.f;
 #pragma unroll
-  for (int k = 0; k < NPL; k++) {
-    const int e = lane * NPL + k;
-    if (e < n) {
-      const float t = sc.hr()[e].t;
-      const float nu = fmaf(b, t, u), nb = fmaf(u, t, b + t);
+    for (int k = 0; k < NPL; k++) {
+      const int e = lane * NPL + k;
+      if (e < n) {
+        const float t = sc.hr()[e].t;
+        const float nu = fmaf(b, t, u), nb = fmaf(u, t, b + t);
+        u = nu;
+        b = nb;
+      }
+    }
+#pragma unroll 1
+    for (int d = 16; d > 0; d >>= 1) {
+      const float ou = __shfl_xor_sync(FULL, u, d), ob = __shfl_xor_sync(FULL, b, d);
+      const float nu = (u + ou) + fmaf(u, ou, b * ob);
+      const float nb = (b + ob) + fmaf(u, ob, b * ou);
       u = nu;
       b = nb;
     }
+    // the butterfly's fused products round differently per lane: take lane
+    // 0's value so the branches below are warp-uniform
+    enz = __shfl_sync(FULL, cls == 0 ? u : (cls == 1 ? b : u + b), 0);
+    if (KEEP) {
+      __syncwarp();
+      if (lane == 0) {
+        kept[0] = 1u;
+        kept[3] = __float_as_uint(enz);
+      }
+      __syncwarp();
+    }
   }
-#pragma unroll 1
-  for (int d = 16; d > 0; d >>= 1) {
-    const float ou = __shfl_xor_sync(FULL, u, d), ob = __shfl_xor_sync(FULL, b, d);
-    const float nu = (u + ou) + fmaf(u, ou, b * ob);
-    const float nb = (b + ob) + fmaf(u, ob, b * ou);
-    u = nu;
-    b = nb;
-  }
-  // the butterfly's fused products round differently per lane: take lane
-  // 0's value so the branches below are warp-uniform
-  const float enz = __shfl_sync(FULL, cls == 0 ? u : (cls == 1 ? b : u + b), 0);
   const float tqf = tq.h + tq.l;
   const float r = enz - tqf;
   if (enz > 0x1p-60f && enz < 0x1p60f) {
     // the hardware log2 (about 2^-22 relative): far inside the soft output's tolerance
     if (r > 0.02f * (enz + tqf)) return {__log2f(r), 0};
     DF E;
-    unsigned *kept = sc.headv() + NPL + 1;
-    if (KEEP && sc.head_at(NPL + 1)) {
+    if (KEEP && (known & 2u) != 0) {
       E = DF{__uint_as_float(sc.head_at(NPL + 2)), __uint_as_float(sc.head_at(NPL + 3))};
     } else {
       E = class_total_df<NPL, SYN>(sc, n, cls, lane);
       if (KEEP) {
         if (lane == 0) {
-          kept[0] = 1u;
+          kept[0] = 3u;
           kept[1] = __float_as_uint(E.h);
           kept[2] = __float_as_uint(E.l);
         }
@@ -1119,8 +1133,18 @@ __device__ int trace_word(const DevCode &code, const Scratch<NPL, SYN> &sc, cons
   return qn;
 }
 
-// threshold rule: predicted probability that the list misses the codeword
+// Threshold rule: whether the predicted probability that the list misses the
+// codeword, e^M / (e^M + sum_l e^lp_l), is below thr.  With s = sum_l
+// e^(lp_l - M) that is thr (1 + s) > 1.  The hardware exponential gives s to
+// about 1e-5, so outside a band of 1e-3 around 1 it decides; inside, the
+// accurate functions do (they took about 60 instructions a list word, at every
+// list word).
 __device__ __forceinline__ bool thr_reached(const float *lp, int nhit, float M, float thr) {
+  float s = 1.f;
+#pragma unroll 1
+  for (int l = 0; l < nhit; l++) s += __expf(lp[l] - M);
+  const float x = thr * s;
+  if (x > 1.001f || x < 0.999f) return x > 1.f;
   float D = M;
 #pragma unroll 1
   for (int l = 0; l < nhit; l++) D = lse(D, lp[l]);
@@ -1255,8 +1279,8 @@ __device__ __forceinline__ void build_prefixes(const Scratch<NPL, SYN> &sc, SYN 
 // lam[k] is bit lane + 32k of the SISO input lambda = fl32(L_Ch + L_A)
 // (the caller loads it; entries past n are ignored).  L_APP is handed to
 // emit(k, x, lapp, listed) for k = 0 .. NPL - 1 in turn: bit lane + 32k, its
-// lambda x and whether the word's list holds a word (else lapp = x).  res gets
-// the per-word results (before the first emit); the list (in query order) is
+// lambda x and whether the word's list holds a word (else lapp = x), after
+// begin().  res gets the per-word results (before the first emit); the list (in query order) is
 // left in the scratch: sc.cw() (codewords, natural bit order), sc.lp() (log
 // p(z)/p(0)) and sc.wl() (APP of each word).  res.flags collects
 // the remaining-mass flags (bit 0: extended range; bit 1: the block's
@@ -1274,9 +1298,9 @@ __device__ __forceinline__ void build_prefixes(const Scratch<NPL, SYN> &sc, SYN 
 // is therefore written for few instructions: lanes share what a single lane
 // could do (list words' APPs, candidates of the 1-line parameter), and loops
 // over the list and over a lane's bits stay rolled.
-template <int NPL, class SYN, int MODE, class Emit>
+template <int NPL, class SYN, int MODE, class Begin, class Emit>
 __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams &P, const Scratch<NPL, SYN> &sc,
-                                          const float (&lam)[NPL], int lane, WordResult &res, Emit emit) {
+                                          const float (&lam)[NPL], int lane, WordResult &res, Begin begin, Emit emit) {
   using LY = Layout<NPL, SYN>;
   constexpr int NM = (32 * NPL + 63) / 64;
   const int n = code.n;
@@ -1290,6 +1314,7 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
   res.queries = -1;
   res.pmiss = 1.f;
   if (!siso_prologue<NPL, SYN>(code, sc, lam, lane, h)) {
+    begin();
 #pragma unroll 1
     for (int k = 0; k < NPL; k++) {
       const float x = sc.lam_at(lane + 32 * k);
@@ -1309,7 +1334,7 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
 #pragma unroll
     for (int k = 0; k < NPL; k++) sc.headv()[k] = h.yb[k];
     sc.headv()[NPL] = (unsigned)h.c;
-    if (MODE == MODE_THR) sc.headv()[NPL + 1] = 0u;  // the class total is not known yet
+    if (MODE == MODE_THR) sc.headv()[NPL + 1] = 0u;  // the class totals are not known yet
   }
   __syncwarp();
   const int tb = __ldg(O.base + ti), tc = __ldg(O.count + ti);
@@ -1532,6 +1557,7 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
   if (lane < nhit) sc.wl()[lane] = wl;
   // eq. LLRi: the miss term, then each listed word adds its APP to the side
   // of its bit
+  begin();
 #pragma unroll 1
   for (int k = 0; k < NPL; k++) {
     const float x = sc.lam_at(lane + 32 * k);
