@@ -265,7 +265,7 @@ int gldpc_decode(sogrand_code *code, int64_t n_frames, const float *llr_ch, int 
 /*
  * Schedule of a code's decoding kernels: 8 (compiled for 8 resident blocks of
  * 128 threads per SM, 64 registers a thread) or 12 (the schedule of more
- * warps: 48 registers a thread, 10 resident blocks).  Which is faster depends
+ * warps: 56 registers a thread, 9 resident blocks).  Which is faster depends
  * on the code (register pressure of its syndrome width and list against the
  * latency the extra warps hide) and is measured by sogrand_code_tune.  The default until tuned: 12 for
  * n <= 64, else 8.

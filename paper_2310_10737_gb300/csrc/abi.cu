@@ -10,6 +10,8 @@
 #include <memory>
 #include <mutex>
 #include <new>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "launch.h"
@@ -85,38 +87,47 @@ struct HostTables {
 // One zone of an order's compact form: entries from `q` on as a prefix slot
 // and the last `ranks` ranks, slots assigned in order of first use, until
 // another slot would be needed, a prefix would not fit its descriptor, or the
-// entries kept end.  The zone stops at a whole group of four chunks.  Returns
-// its end.
-int compact_zone(const uint4 *ent, int q, int count, int n, int ranks, int max_slots, uint2 *slots,
-                 std::vector<uint32_t> &out) {
+// entries kept end.  The zone stops at a whole group of four chunks.  Writes
+// query 128 g + 32 c + j as lane j's c-th entry of group g; returns the zone's
+// end.  No allocation (it runs on helper threads).
+int compact_zone(const uint4 *ent, int q, int count, int n, int ranks, int max_slots, uint2 *slots, uint32_t *dst) {
   // open-addressed table of the slots in use, keyed by their descriptor
-  int table[256];
-  std::fill(table, table + 256, -1);
-  int used = 0;
+  uint64_t keys[256];
+  int16_t slot_of[256];
+  std::fill(slot_of, slot_of + 256, (int16_t)-1);
+  int used = 0, last = -1;
+  uint64_t last_key = 0;
   const int start = q;
   for (; q < count; q++) {
-    uint8_t b[16];
-    std::memcpy(b, ent + q, 16);
-    const int w = b[0], rest = std::min(w, ranks), len = w - rest;
+    uint64_t lo, hi;  // the entry's bytes: weight, then the ranks
+    std::memcpy(&lo, &ent[q].x, 8);
+    std::memcpy(&hi, &ent[q].z, 8);
+    const int w = (int)(lo & 0xff), rest = std::min(w, ranks), len = w - rest;
     if (len > sg::FAST_PREFIX) break;
-    uint8_t d[8] = {(uint8_t)(len | (rest << 4)), 0, 0, 0, 0, 0, 0, 0};
-    for (int i = 0; i < len; i++) d[1 + i] = b[1 + i];
-    uint64_t key;
-    std::memcpy(&key, d, 8);
-    unsigned at = (unsigned)((key * 0x9E3779B97F4A7C15ull) >> 56);
-    while (table[at] >= 0 && std::memcmp(&slots[table[at]], d, 8) != 0) at = (at + 1) & 255;
-    if (table[at] < 0) {
-      if (used == max_slots) break;
-      std::memcpy(&slots[used], d, 8);
-      table[at] = used++;
+    // descriptor: byte 0 the lengths, then the prefix's ranks
+    const uint64_t mask = len == 7 ? ~0ull : (1ull << (8 * (len + 1))) - 1;
+    const uint64_t key = ((lo & mask) & ~0xffull) | (uint64_t)(len | (rest << 4));
+    if (last < 0 || key != last_key) {  // neighbours often share their prefix
+      unsigned at = (unsigned)((key * 0x9E3779B97F4A7C15ull) >> 56);
+      while (slot_of[at] >= 0 && keys[at] != key) at = (at + 1) & 255;
+      if (slot_of[at] < 0) {
+        if (used == max_slots) break;
+        std::memcpy(&slots[used], &key, 8);
+        keys[at] = key;
+        slot_of[at] = (int16_t)used++;
+      }
+      last = slot_of[at];
+      last_key = key;
     }
-    uint32_t e = (uint32_t)table[at];
-    for (int i = 0; i < 3; i++) e |= (uint32_t)(i < rest ? b[1 + len + i] : n) << (8 + 8 * i);
-    out.push_back(e);
+    uint32_t e = (uint32_t)last;
+    for (int i = 0; i < 3; i++) {
+      const int by = 1 + len + i;  // at most 10
+      const uint32_t r = (uint32_t)((by < 8 ? lo >> (8 * by) : hi >> (8 * (by - 8))) & 0xff);
+      e |= (i < rest ? r : (uint32_t)n) << (8 + 8 * i);
+    }
+    dst[(q & ~127) + 4 * (q & 31) + ((q >> 5) & 3)] = e;
   }
-  const int end = start + ((q - start) & ~127);
-  out.resize(out.size() - (size_t)(q - end));
-  return end;
+  return start + ((q - start) & ~127);
 }
 
 // cnt[w][m] = number of w-subsets of {1..n} with sum m (saturating), w <= wlim
@@ -242,27 +253,34 @@ int build_tables(int n, int64_t cap, int c_max, bool even, HostTables &T) {
       T.count[(size_t)c * ncls + K] = (int32_t)(T.ent.size() - start);
     }
   }
-  // the compact forms of every order's head
+  // the compact forms of every order's head, built by a few threads (a
+  // million entries for n = 64: 20 ms on one)
   const int orders = (c_max + 1) * ncls, per = sg::FAST_SLOTS2 + sg::FAST_SLOTS;
   T.slots.assign((size_t)orders * per, make_uint2(0, 0));
   T.zones.assign(orders, make_int2(0, 0));
-  std::vector<std::vector<uint32_t>> heads(orders);
-  int longest = 0;
-  for (int ti = 0; ti < orders; ti++) {
-    const uint4 *ent = &T.ent[T.base[ti]];
-    const int count = std::min(T.count[ti], sg::FAST_QUERIES);
-    int2 &z = T.zones[ti];
-    z.x = compact_zone(ent, 0, count, n, 2, sg::FAST_SLOTS2, &T.slots[(size_t)ti * per], heads[ti]);
-    z.y = compact_zone(ent, z.x, count, n, 3, sg::FAST_SLOTS, &T.slots[(size_t)ti * per + sg::FAST_SLOTS2], heads[ti]);
-    longest = std::max(longest, z.y);
-  }
-  T.e4_stride = longest / 4 + 64;  // padded: two groups past the head are read ahead
+  const int most = std::min(*std::max_element(T.count.begin(), T.count.end()), sg::FAST_QUERIES);
+  T.e4_stride = (most + 127) / 128 * 32 + 64;  // padded: two groups past the head are read ahead
   T.e4.assign((size_t)orders * T.e4_stride, make_uint4(0u, 0u, 0u, 0u));
-  for (int ti = 0; ti < orders; ti++) {
-    uint32_t *dst = &T.e4[(size_t)ti * T.e4_stride].x;
-    for (size_t q = 0; q < heads[ti].size(); q++)  // query 128 g + 32 c + j: lane j's c-th entry of group g
-      dst[(q & ~size_t(127)) + 4 * (q & 31) + ((q >> 5) & 3)] = heads[ti][q];
+  std::atomic<int> next{0};
+  const auto work = [&]() {
+    for (int ti = next++; ti < orders; ti = next++) {
+      const uint4 *ent = T.ent.data() + T.base[ti];
+      const int count = std::min(T.count[ti], sg::FAST_QUERIES);
+      uint2 *slots = &T.slots[(size_t)ti * per];
+      uint32_t *dst = &T.e4[(size_t)ti * T.e4_stride].x;
+      int2 &z = T.zones[ti];
+      z.x = compact_zone(ent, 0, count, n, 2, sg::FAST_SLOTS2, slots, dst);
+      z.y = compact_zone(ent, z.x, count, n, 3, sg::FAST_SLOTS, slots + sg::FAST_SLOTS2, dst);
+    }
+  };
+  std::vector<std::thread> helpers;
+  helpers.reserve(7);
+  try {
+    for (unsigned i = 1; i < std::min(8u, std::thread::hardware_concurrency()); i++) helpers.emplace_back(work);
+  } catch (const std::system_error &) {  // no more threads: this one does the rest
   }
+  work();
+  for (std::thread &t : helpers) t.join();
   T.jmax = maxcost + 2;
   T.gbase.push_back((int32_t)T.grp.size());
   // scnt[N][w][m]: w-subsets of {1..N} with sum m (N = 0..n, w < sc_w, m <= the
@@ -583,7 +601,7 @@ int sogrand_code_create(int n, int k, const uint8_t *H, int even, sogrand_code *
   c->even = even;
   c->c_max = n;
   c->nm = (n + 63) / 64;
-  // default schedule until tuned: 12 (10 blocks per SM, 48 registers) for codes
+  // default schedule until tuned: 12 (9 blocks per SM, 56 registers) for codes
   // of up to 64 bits, else 8 (64 registers)
   c->minb = n <= 64 ? 12 : 8;
   // and the remaining-mass area in global memory for the others (they gain L1)
@@ -841,7 +859,7 @@ size_t persistent_scratch_bytes(int64_t F, int nr, int nc, int nm, int max_iter)
 }
 
 // The global remaining-mass region of a persistent launch: one slice per
-// resident block (at most 8 blocks per SM in either schedule).
+// resident block (at most MAX_BLOCKS_PER_SM an SM in either schedule).
 inline int npl_of_n(int n) { return n <= 32 ? 1 : (n <= 64 ? 2 : 4); }
 int dp_slice_of(const sogrand_code *rc, const sogrand_code *cc) {
   return sg::dp_slice_bytes(npl_of_n(rc->n), rc->m > 32 ? 8 : 4, std::max(rc->jmax, cc->jmax));

@@ -23,10 +23,11 @@ constexpr int TPB = 32 * WARPS_PER_BLOCK;
 
 // Resident blocks per SM that a schedule's kernels are compiled for.  Schedule
 // 8 takes 64 registers a thread; schedule 12 (its name: the second value of
-// sogrand_code_schedule) 48 registers, which is 10 blocks: at 40 (12 blocks)
-// the word's code spills and grows by 10%, and the two blocks more leave less
-// L1 (eBCH(64,57)^2, 20,000 frames: 27.0 ms at 10 blocks, 27.9 at 12).
-__host__ __device__ constexpr int resident_blocks(int minb) { return minb == 12 ? 10 : minb; }
+// sogrand_code_schedule) 56 registers, which is 9 blocks.  The launch is bound
+// by issue and the instruction cache, not by latency that more warps would
+// hide, and more blocks leave less L1 (eBCH(64,57)^2, 20,000 frames: 21.0 ms
+// at 7 blocks, 20.3 at 8, 20.1 at 9, 21.3 at 10; at 12 the code also spills).
+__host__ __device__ constexpr int resident_blocks(int minb) { return minb == 12 ? 9 : minb; }
 
 // The warp's index in its block, broadcast so that the compiler knows it to be
 // the same in every lane: the words' control flow is then provably uniform
@@ -106,7 +107,7 @@ __global__ void __launch_bounds__(TPB, resident_blocks(MINB)) k_decode(const __g
       lam[k] = x;
     }
     WordResult res;
-    siso_word<NPL, SYN, MODE>(code, P, sc, lam, lane, res, [] {}, [&](int k, float x, float lapp, bool listed) {
+    siso_word<NPL, SYN, MODE, true>(code, P, sc, lam, lane, res, [] {}, [&](int k, float x, float lapp, bool listed) {
       const int i = lane + 32 * k;
       if (i < n) {
         if (a.llr_app) a.llr_app[base + i] = lapp;
@@ -261,7 +262,7 @@ __device__ __forceinline__ int product_word(const DevCode &code, const SisoParam
   float *le = nullptr;
   unsigned *hb = nullptr;
   size_t at = 0;
-  siso_word<NPL, SYN, MODE>(
+  siso_word<NPL, SYN, MODE, false>(
       code, P, sc, lam, lane, res,
       [&]() {
         f = vc->f;
@@ -573,7 +574,8 @@ __device__ __forceinline__ int32_t slot_value(int li, int half) {
 __device__ __forceinline__ int sched_wait(const ProductArgs &a, int slot, int lane, int *waited) {
   const bool real = slot < a.n_frames * a.max_half;  // a frame has at most max_half halves
   int v = 0;
-  unsigned slept = 0, nap = 64;  // slept: microseconds / 1.024
+  long long slept = 0;  // nanoseconds
+  unsigned nap = 64;
   for (;;) {
     int stop = 0;
     if (lane == 0) {
@@ -590,7 +592,7 @@ __device__ __forceinline__ int sched_wait(const ProductArgs &a, int slot, int la
     if (stop) return 0;
     if (v != 0) break;
     *waited = 1;
-    if ((slept >> 10) > (unsigned)a.max_spin) {
+    if (slept > (long long)a.max_spin * 1000) {
       if (lane == 0) atomicExch(a.ctrl + CTRL_ERROR, 1);
       return 0;
     }
@@ -817,7 +819,7 @@ inline int grid_for(K kernel, int smem, int64_t warps_needed) {
 }
 
 // The schedule a launch runs: the code's, except that schedule 12's kernels
-// (48 registers) are used only when the launch has more words than the 8-block
+// (56 registers) are used only when the launch has more words than the 8-block
 // grid has warps; a smaller batch gains nothing from the extra warps and
 // decodes each word faster at 64 registers.
 inline int launch_minb(int minb, int64_t words) {

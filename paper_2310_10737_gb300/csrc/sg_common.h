@@ -13,9 +13,9 @@ constexpr int WMAXT = 64;      // most Hamming weights a query-order table may r
 constexpr int WENT = 15;       // most ranks one table entry holds
 constexpr int WARPS_PER_BLOCK = 4;
 // Schedules: the per-word kernels are compiled for 8 resident blocks per SM
-// (64 registers a thread, schedule 8) and for 10 (48 registers, schedule 12); a
+// (64 registers a thread, schedule 8) and for 9 (56 registers, schedule 12); a
 // launch never has more than MAX_BLOCKS_PER_SM blocks resident on an SM.
-constexpr int MAX_BLOCKS_PER_SM = 12;
+constexpr int MAX_BLOCKS_PER_SM = 9;
 
 // Query order of one code, flattened per 1-line parameter c and parity class.
 // For every c in [0, c_max] and class (the parity of y for an even code, or

@@ -126,12 +126,12 @@ __device__ __forceinline__ void df_acc(DF &a, DF x) {
   a.h = s;
   a.l = __fadd_rn(a.l, __fadd_rn(err, x.l));
 }
-// The warp butterflies that run once per word are loops, not unrolled: the
-// kernel's per-word path is long and instruction fetch is its first stall, so
-// a smaller path is faster (these three loops: 7% for eBCH(64,57)).
+// The warp butterflies that run once per word are loops, unrolled only where
+// the kernel's code leaves room in the instruction cache (ROOMY, siso_word).
+template <bool ROOMY>
 __device__ __forceinline__ DF df_warp_sum(DF x) {  // x >= 0; lane 0's result broadcast (warp-uniform)
   x = df_norm(x.h, x.l);
-#pragma unroll 1
+#pragma unroll(ROOMY ? 5 : 1)
   for (int d = 16; d > 0; d >>= 1)
     x = df_add_pos(x, DF{__shfl_xor_sync(0xffffffffu, x.h, d), __shfl_xor_sync(0xffffffffu, x.l, d)});
   return {__shfl_sync(0xffffffffu, x.h, 0), __shfl_sync(0xffffffffu, x.l, 0)};
@@ -810,7 +810,7 @@ __device__ __forceinline__ Remaining remaining_log2_dp(const Scratch<NPL, SYN> &
 // few 2^-46 moves it by at most about 1e-5 relative).  Otherwise the
 // unqueried patterns are summed directly.  KEEP: the class totals are kept
 // with the word's head (the threshold rule asks at every listed word).
-template <bool KEEP, int NPL, class SYN>
+template <bool KEEP, bool ROOMY, int NPL, class SYN>
 __device__ __forceinline__ Remaining remaining_log2(const Scratch<NPL, SYN> &sc, const uint4 *ent,
                                                     const uint16_t *cost, int tc, int qs, int n, int cls, int lane,
                                                     DF tq) {
@@ -832,7 +832,7 @@ __device__ __forceinline__ Remaining remaining_log2(const Scratch<NPL, SYN> &sc,
         b = nb;
       }
     }
-#pragma unroll 1
+#pragma unroll(ROOMY ? 5 : 1)
     for (int d = 16; d > 0; d >>= 1) {
       const float ou = __shfl_xor_sync(FULL, u, d), ob = __shfl_xor_sync(FULL, b, d);
       const float nu = (u + ou) + fmaf(u, ou, b * ob);
@@ -1297,8 +1297,11 @@ __device__ __forceinline__ void build_prefixes(const Scratch<NPL, SYN> &sc, SYN 
 // competes for the SM's instruction cache.  Everything that runs once per word
 // is therefore written for few instructions: lanes share what a single lane
 // could do (list words' APPs, candidates of the 1-line parameter), and loops
-// over the list and over a lane's bits stay rolled.
-template <int NPL, class SYN, int MODE, class Begin, class Emit>
+// over the list and over a lane's bits stay rolled.  ROOMY: the kernel has
+// little other code (k_decode), and the per-word sums are unrolled (2% faster
+// there; in the batched kernel they pushed the code past the instruction cache,
+// 4% slower).
+template <int NPL, class SYN, int MODE, bool ROOMY, class Begin, class Emit>
 __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams &P, const Scratch<NPL, SYN> &sc,
                                           const float (&lam)[NPL], int lane, WordResult &res, Begin begin, Emit emit) {
   using LY = Layout<NPL, SYN>;
@@ -1519,8 +1522,8 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
     Remaining rem = {-CUDART_INF_F, 0};
     // when the whole parity class has been queried nothing remains
     if (!(fin && qn >= tc && tc == O.class_size) && !P.forney)
-      rem = remaining_log2<MODE == MODE_THR, NPL, SYN>(sc, ent, O.cost + tb, tc, qn - 1, n, cls, lane,
-                                                       df_warp_sum(part));
+      rem = remaining_log2<MODE == MODE_THR, ROOMY, NPL, SYN>(sc, ent, O.cost + tb, tc, qn - 1, n, cls, lane,
+                                                       df_warp_sum<ROOMY>(part));
     res.flags |= rem.flags;
     M = fmaf(rem.lr2, LN2_F, code.log_phi);
     if (MODE != MODE_THR || fin || thr_reached(sc.lp(), nhit, M, P.thr)) {
@@ -1558,7 +1561,7 @@ __device__ __forceinline__ void siso_word(const DevCode &code, const SisoParams 
   // eq. LLRi: the miss term, then each listed word adds its APP to the side
   // of its bit
   begin();
-#pragma unroll 1
+#pragma unroll(ROOMY ? NPL : 1)
   for (int k = 0; k < NPL; k++) {
     const float x = sc.lam_at(lane + 32 * k);
     // sigma(x) and sigma(-x) without cancellation
