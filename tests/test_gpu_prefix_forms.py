@@ -56,3 +56,58 @@ def test_forms_match_oracle(oracle_lib, name, cap, L, thr, even):
     c.close()
     ref = oracle_lib.siso_batch(oracle_lib.OracleCode(lc), lch, L=L, cap=cap, thr=thr)
     compare_siso(lc, out, ref, f"{name} cap={cap} L={L} thr={thr}")
+
+
+@pytest.mark.parametrize("name", ["ebch_16_11", "ebch_32_26", "ebch_64_57", "ebch_128_120"])
+def test_order_of_nearly_equal_reliabilities(oracle_lib, name):
+    """The reliability sort drops the lowest bits of |lambda| from its keys and
+    restores the exact order afterwards: values a few units in the last place
+    apart (and equal ones, which fall to the lower index), whole words of them
+    and a few among ordinary ones, must give the oracle's queries and lists."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2310_10737_gb300 as sg
+    lc = ebch(name)
+    rng = np.random.default_rng(12)
+    W = 200
+    near = np.float32(2.0) + rng.integers(0, 40, (W, lc.n)).astype(np.float32) * np.float32(2.0 ** -22)
+    lch = near * rng.choice(np.array([-1.0, 1.0], np.float32), (W, lc.n))
+    some = rng.random((W, lc.n)) < 0.8  # from word 100 on, most values are ordinary
+    some[:100] = False
+    lch = np.where(some, rng.standard_normal((W, lc.n)) * 4.0, lch).astype(np.float32)
+    c = sg.Code.from_linear_code(lc)
+    out = sg.sogrand_decode(c, torch.from_numpy(lch).cuda(), L=4, query_cap=3000)
+    torch.cuda.synchronize()
+    c.close()
+    ref = oracle_lib.siso_batch(oracle_lib.OracleCode(lc), lch, L=4, cap=3000)
+    compare_siso(lc, out, ref, f"{name} near ties")
+
+
+@pytest.mark.parametrize("row,col,frames", [("ebch_16_11", "ebch_32_26", 1), ("ebch_16_11", "ebch_32_26", 3500),
+                                            ("ebch_32_26", "ebch_16_11", 6001), ("ebch_32_26", "ebch_32_26", 12003),
+                                            ("ebch_16_11", "ebch_16_11", 12001)])
+def test_ticket_runs_equal_plain_form(row, col, frames):
+    """Batches small and large enough that warps draw one, two, four or eight
+    word tickets at once (5,472 warps: 8, 16, 32 and 64 words each), with halves
+    that leave tickets unused: every output as the plain form gives it."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2310_10737_gb300 as sg
+    from workloads import awgn_frames
+    r, c = ebch(row), ebch(col)
+    _, _, llr = awgn_frames(r, min(frames, 1500), 2.5, seed=5, col_code=c, threads=8)
+    llr = np.tile(llr, (-(-frames // len(llr)), 1, 1))[:frames]
+    d = torch.from_numpy(np.ascontiguousarray(llr)).cuda()
+    kr, kc = sg.Code.from_linear_code(r), sg.Code.from_linear_code(c)
+    kc = kr if row == col else kc
+    a = sg.product_decode(kr, d, max_iter=6, col_code=kc)
+    b = sg.product_decode(kr, d, max_iter=6, col_code=kc, persistent=True)
+    torch.cuda.synchronize()
+    for key in ("bits", "half_iters", "status", "queries", "par_queries", "weight_sum"):
+        assert torch.equal(a[key], b[key]), key
