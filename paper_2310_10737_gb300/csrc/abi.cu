@@ -7,10 +7,10 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <memory>
 #include <mutex>
 #include <new>
-#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -277,7 +277,7 @@ int build_tables(int n, int64_t cap, int c_max, bool even, HostTables &T) {
   helpers.reserve(7);
   try {
     for (unsigned i = 1; i < std::min(8u, std::thread::hardware_concurrency()); i++) helpers.emplace_back(work);
-  } catch (const std::system_error &) {  // no more threads: this one does the rest
+  } catch (const std::exception &) {  // no more threads (or no memory for one): this thread does the rest
   }
   work();
   for (std::thread &t : helpers) t.join();
