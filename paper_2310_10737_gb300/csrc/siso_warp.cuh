@@ -383,8 +383,8 @@ __device__ __forceinline__ void warp_sort_blocked(unsigned (&v)[NPL], int lane) 
 
 // Exact order of the rank records where truncated keys left neighbours
 // descending: odd-even transposition on |lambda| (equal values keep their
-// order, the lower bit first).  About 0.5% of 64-bit words need it, a pass or
-// two each.
+// order, the lower bit first).  0.02%, 0.16% and 1.3% of 32-, 64- and 128-bit
+// words at 3 dB need it, a pass or two each.
 template <int NPL>
 __device__ __forceinline__ void fix_rank_order(RankBit *rb, int n, int lane) {
   int moved;
