@@ -585,6 +585,11 @@ __device__ __forceinline__ void dp_ranks(int Cs, int c, int R0, int cls, const t
 // The (scaled) remaining mass summed over the warp.  With FOps every mass
 // carries the factor 2^(g2 * Cs) (g2 = gamma log2 e); with XOps g2 = 0.
 // `ent` and `cost` are the word's order, `tc` its entries, `qs` the last queried pattern.
+// The products with g2 are rounded by themselves (__fmul_rn): left to the
+// compiler, each kernel that this is inlined into fused some of them with the
+// subtraction that follows, and the same word's mass came out differently with
+// and without the threshold rule (by a unit or two in the last place of its
+// logarithm).
 template <class Ops, int NPL, class SYN>
 __device__ __forceinline__ typename Ops::T remaining_scaled(const Scratch<NPL, SYN> &sc, const uint4 *ent,
                                                             const uint16_t *cost, int tc, int qs, int n, int c,
@@ -599,7 +604,7 @@ __device__ __forceinline__ typename Ops::T remaining_scaled(const Scratch<NPL, S
   T *ho = he + (Cs + 1);
   constexpr bool SCALED = sizeof(T) == 4;
   const int R0 = min(max(Cs - c, 0), n);  // ranks e < R0 can sit inside a pattern of cost <= Cs
-  const float g2Cs = g2 * (float)Cs;
+  const float g2Cs = __fmul_rn(g2, (float)Cs);
 
   // --- unqueried rest of level Cs (the table stores every level completely)
   T acc = Ops::zero();
@@ -610,7 +615,7 @@ __device__ __forceinline__ typename Ops::T remaining_scaled(const Scratch<NPL, S
     if (in) {
       const uint4 e = __ldg(ent + q);
       const float s2 = ent_sum<NPL, SYN>(e, e.x & 0xff, sc);
-      acc = Ops::add(acc, Ops::from_log2(g2Cs - s2));
+      acc = Ops::add(acc, Ops::from_log2(__fsub_rn(g2Cs, s2)));
     }
     if (!__all_sync(FULL, in)) break;  // costs are nondecreasing
   }
@@ -629,7 +634,7 @@ __device__ __forceinline__ typename Ops::T remaining_scaled(const Scratch<NPL, S
         t = Ops::from_log2(-sc.l2(e));
         // factor used by the tail: low ranks t * 2^(g2 d_e), high ranks t * 2^(g2 Cs)
         const float d = (float)(e + 1 + c);
-        sfac[e] = Ops::from_log2((e < R0 ? g2 * d : g2Cs) - sc.l2(e));
+        sfac[e] = Ops::from_log2(__fsub_rn(e < R0 ? __fmul_rn(g2, d) : g2Cs, sc.l2(e)));
       }
       const T nu = Ops::fma(b, t, u);
       const T nb = Ops::fma(u, t, Ops::add(b, t));
@@ -787,7 +792,7 @@ __device__ __forceinline__ Remaining remaining_log2_dp(const Scratch<NPL, SYN> &
   const float tot =
       __shfl_sync(FULL, remaining_scaled<FOps, NPL, SYN>(sc, ent, cost, tc, qs, n, c, cls, Cs, g, lane), 0);
   if (tot >= 0x1p-60f && tot < CUDART_INF_F) {
-    out.lr2 = log2f(tot) - g * (float)Cs;
+    out.lr2 = fmaf(-g, (float)Cs, log2f(tot));  // one rounding of a difference of two large terms
   } else {
     out.flags = 1;
 #ifdef SG_PHASE_PROFILE
