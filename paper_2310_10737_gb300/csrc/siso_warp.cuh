@@ -1141,15 +1141,17 @@ __device__ int trace_word(const DevCode &code, const Scratch<NPL, SYN> &sc, cons
 // Threshold rule: whether the predicted probability that the list misses the
 // codeword, e^M / (e^M + sum_l e^lp_l), is below thr.  With s = sum_l
 // e^(lp_l - M) that is thr (1 + s) > 1.  The hardware exponential gives s to
-// about 1e-5, so outside a band of 1e-3 around 1 it decides; inside, the
-// accurate functions do (they took about 60 instructions a list word, at every
-// list word).
+// about 1e-5, so outside a band around 1 it decides; inside, the accurate
+// functions do (they took about 60 instructions a list word, at every list
+// word).  Their sum is taken in the log domain and is itself off by up to an
+// ulp of M a list word (16 of them: 1e-6 |M|), so the band grows with |M|.
 __device__ __forceinline__ bool thr_reached(const float *lp, int nhit, float M, float thr) {
   float s = 1.f;
 #pragma unroll 1
   for (int l = 0; l < nhit; l++) s += __expf(lp[l] - M);
   const float x = thr * s;
-  if (x > 1.001f || x < 0.999f) return x > 1.f;
+  const float band = fmaf(fabsf(M), 2e-6f, 1e-3f);
+  if (x > 1.f + band || x < 1.f - band) return x > 1.f;
   float D = M;
 #pragma unroll 1
   for (int l = 0; l < nhit; l++) D = lse(D, lp[l]);
