@@ -1145,12 +1145,14 @@ __device__ int trace_word(const DevCode &code, const Scratch<NPL, SYN> &sc, cons
 // functions do (they took about 60 instructions a list word, at every list
 // word).  Their sum is taken in the log domain and is itself off by up to an
 // ulp of M a list word (16 of them: 1e-6 |M|), so the band grows with |M|.
+// Thresholds below the smallest normal number, where s overflows and the
+// probability is a denormal, are left to them altogether.
 __device__ __forceinline__ bool thr_reached(const float *lp, int nhit, float M, float thr) {
   float s = 1.f;
 #pragma unroll 1
   for (int l = 0; l < nhit; l++) s += __expf(lp[l] - M);
   const float x = thr * s;
-  const float band = fmaf(fabsf(M), 2e-6f, 1e-3f);
+  const float band = thr >= 0x1p-126f ? fmaf(fabsf(M), 2e-6f, 1e-3f) : CUDART_INF_F;
   if (x > 1.f + band || x < 1.f - band) return x > 1.f;
   float D = M;
 #pragma unroll 1

@@ -38,3 +38,22 @@ def test_large_masses(env, name, mean, spread, queries):
     torch.cuda.synchronize()
     c.close()
     assert out["queries"].tolist() == list(queries.values())
+
+
+@pytest.mark.parametrize("name", ["ebch_32_26", "ebch_64_57", "ebch_128_120"])
+@pytest.mark.parametrize("thr", [1e-37, 1e-40, 1e-42])
+def test_denormal_thresholds(env, oracle_lib, name, thr):
+    """Clean words whose miss probability is near 1e-39: a threshold of 1e-37
+    stops them at the first list word, a denormal one does not (the quick sum
+    overflows there)."""
+    torch, sg = env
+    lc = ebch(name)
+    x = (45 + np.random.default_rng(3).integers(0, 1280, (40, lc.n)) / 256).astype(np.float32)
+    c = sg.Code.from_linear_code(lc)
+    out = sg.sogrand_decode(c, torch.from_numpy(x).cuda(), L=2, query_cap=2000, thr=thr)
+    torch.cuda.synchronize()
+    c.close()
+    ref = oracle_lib.siso_batch(oracle_lib.OracleCode(lc), x, L=2, cap=2000, thr=float(np.float32(thr)))
+    assert (ref["queries"] == 1).all() == (thr > 1e-38)
+    np.testing.assert_array_equal(out["queries"].cpu().numpy(), ref["queries"])
+    np.testing.assert_array_equal(out["list_count"].cpu().numpy(), ref["list_count"])
