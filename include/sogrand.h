@@ -91,7 +91,10 @@ int sogrand_code_tables(const sogrand_code *code, int64_t *query_cap, int64_t *b
  *   queue_wait_us  microseconds of accumulated back-off that a warp of a
  *                  batched (persistent) launch waits for work before the
  *                  launch stops and returns SOGRAND_ETIMEOUT (default
- *                  2,000,000; 0 gives up at the first wait)
+ *                  2,000,000; 0 gives up at the first wait).  It has to
+ *                  cover the longest search of a word under the query cap; in
+ *                  a large batch, where a warp takes 2, 4 or 8 words at once,
+ *                  the launch waits 2, 4 or 8 times as long
  *   lock_polls     polls of its block's remaining-mass lock after which a
  *                  warp gives up on the lock (default 2^22); the batched forms
  *                  then stop and return SOGRAND_ETIMEOUT
@@ -230,7 +233,8 @@ int product_decode_ex(sogrand_code *row_code, const sogrand_code *col_code, int6
  * the frame or queues it for its next half.  No per-half launches and no
  * host round trips; every frame advances at its own pace.  Waits inside the
  * kernel are bounded (sogrand_set_wait_limits): if a warp finds no work for
- * 2 s of accumulated back-off while frames are unfinished, or cannot take its
+ * 2 s of accumulated back-off (up to 16 s in a batch of 64 words a warp or
+ * more) while frames are unfinished, or cannot take its
  * block's remaining-mass lock, the kernel stops and the call returns
  * SOGRAND_ETIMEOUT.  stats->timing_ms[0] is the kernel's device time;
  * launches counts 2 (queue set-up and the decoder).  Scratch, allocated

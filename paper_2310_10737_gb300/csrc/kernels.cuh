@@ -568,7 +568,9 @@ __device__ __forceinline__ int32_t slot_value(int li, int half) {
 // Wait until slot `slot` of the frame-half list is filled.  Returns its signed
 // value, or 0 when the list is done (every frame finished or parked) or the
 // launch's error word is set.  The wait backs off exponentially and gives up
-// after max_spin microseconds of sleep, setting the error word.  All reads of
+// after max_spin microseconds of sleep for every word that a warp draws at
+// once (what it waits for may be all the words of another warp's run, decoded
+// one after the other), setting the error word.  All reads of
 // shared state are made by lane 0 and broadcast, so the whole warp takes the
 // same branch.
 __device__ __forceinline__ int sched_wait(const ProductArgs &a, int slot, int lane, int *waited) {
@@ -592,7 +594,7 @@ __device__ __forceinline__ int sched_wait(const ProductArgs &a, int slot, int la
     if (stop) return 0;
     if (v != 0) break;
     *waited = 1;
-    if (slept > (long long)a.max_spin * 1000) {
+    if (slept > (long long)a.max_spin * 1000 * a.run) {
       if (lane == 0) atomicExch(a.ctrl + CTRL_ERROR, 1);
       return 0;
     }
@@ -652,7 +654,7 @@ __device__ __forceinline__ void frame_after_half(const DevCode &wc, const DevCod
 // A warp whose slot is not filled yet waits with exponential back-off (the
 // tickets of its run then lie in slots that are not reserved yet or about to be
 // stored, so it holds back no word that another warp waits for); all waits are
-// bounded (a.max_spin microseconds of accumulated sleep without progress):
+// bounded (a.max_spin * a.run microseconds of accumulated sleep without progress):
 // the kernel then records an error and every warp returns.  GEN: two codes or
 // wrapped diagonals (the code of a word is chosen per half); otherwise a
 // square product code whose words all use rowc, with no per-word selection

@@ -55,7 +55,7 @@ struct ProductArgs {
   int32_t *bad;               // [F] a non-finite input was seen
   int32_t *ctrl;              // [CTRL_WORDS] the scheduler's words, indexed by CTRL_*
   int32_t run;                // word tickets a warp draws at once while the list runs ahead of it
-  int32_t max_spin;           // microseconds of accumulated back-off without work before giving up
+  int32_t max_spin;           // microseconds of accumulated back-off without work before giving up, times run
   int32_t *half_stop;         // [F] or null: park the frame after this half (serving epochs)
   // serving: the launch decodes the frames named by a list (buffer indices;
   // an entry -(f + 1) marks frame f as newly admitted: its counters are
