@@ -7,11 +7,10 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
-#include <exception>
 #include <memory>
 #include <mutex>
 #include <new>
-#include <thread>
+#include <utility>
 #include <vector>
 
 #include "launch.h"
@@ -84,49 +83,83 @@ struct HostTables {
   int e4_stride = 0;
 };
 
-// One zone of an order's compact form: entries from `q` on as a prefix slot
-// and the last `ranks` ranks, slots assigned in order of first use, until
-// another slot would be needed, a prefix would not fit its descriptor, or the
-// entries kept end.  The zone stops at a whole group of four chunks.  Writes
-// query 128 g + 32 c + j as lane j's c-th entry of group g; returns the zone's
-// end.  No allocation (it runs on helper threads).
-int compact_zone(const uint4 *ent, int q, int count, int n, int ranks, int max_slots, uint2 *slots, uint32_t *dst) {
-  // open-addressed table of the slots in use, keyed by their descriptor
-  uint64_t keys[256];
-  int16_t slot_of[256];
-  std::fill(slot_of, slot_of + 256, (int16_t)-1);
-  int used = 0, last = -1;
-  uint64_t last_key = 0;
-  const int start = q;
-  for (; q < count; q++) {
+// The patterns of one weight split into a prefix and their last ranks, for one
+// of the compact forms: the same for every order, so it is done once.
+struct SplitStream {
+  std::vector<uint2> part;    // per pattern: number of its prefix; last ranks in bytes 1..3
+  std::vector<uint2> desc;    // per prefix: its descriptor (DevOrder::slots)
+  std::vector<int16_t> slot;  // per prefix: its slot in the zone being laid down, or -1
+};
+
+// Split the first `count` patterns of weight w (none when a prefix would not
+// fit its descriptor).  Bytes past a pattern's ranks hold n already.
+SplitStream split_stream(const std::vector<uint4> &stream, int count, int w, int ranks) {
+  SplitStream S;
+  const int rest = std::min(w, ranks), len = w - rest;
+  if (len > sg::FAST_PREFIX) return S;
+  S.part.reserve(count);
+  const uint64_t mask = (len == 7 ? ~0ull : (1ull << (8 * (len + 1))) - 1) & ~0xffull;
+  int lg = 6;
+  while ((1 << lg) < 2 * count) lg++;
+  std::vector<int> at((size_t)1 << lg, -1);  // open-addressed: prefixes by descriptor
+  std::vector<uint64_t> keys;
+  int last = -1;
+  for (int i = 0; i < count; i++) {
     uint64_t lo, hi;  // the entry's bytes: weight, then the ranks
-    std::memcpy(&lo, &ent[q].x, 8);
-    std::memcpy(&hi, &ent[q].z, 8);
-    const int w = (int)(lo & 0xff), rest = std::min(w, ranks), len = w - rest;
-    if (len > sg::FAST_PREFIX) break;
+    std::memcpy(&lo, &stream[i].x, 8);
+    std::memcpy(&hi, &stream[i].z, 8);
     // descriptor: byte 0 the lengths, then the prefix's ranks
-    const uint64_t mask = len == 7 ? ~0ull : (1ull << (8 * (len + 1))) - 1;
-    const uint64_t key = ((lo & mask) & ~0xffull) | (uint64_t)(len | (rest << 4));
-    if (last < 0 || key != last_key) {  // neighbours often share their prefix
-      unsigned at = (unsigned)((key * 0x9E3779B97F4A7C15ull) >> 56);
-      while (slot_of[at] >= 0 && keys[at] != key) at = (at + 1) & 255;
-      if (slot_of[at] < 0) {
-        if (used == max_slots) break;
-        std::memcpy(&slots[used], &key, 8);
-        keys[at] = key;
-        slot_of[at] = (int16_t)used++;
+    const uint64_t key = (lo & mask) | (uint64_t)(len | (rest << 4));
+    if (last < 0 || keys[last] != key) {  // neighbours often share their prefix
+      size_t h = (size_t)((key * 0x9E3779B97F4A7C15ull) >> (64 - lg));
+      while (at[h] >= 0 && keys[at[h]] != key) h = (h + 1) & (((size_t)1 << lg) - 1);
+      if (at[h] < 0) {
+        at[h] = (int)keys.size();
+        keys.push_back(key);
       }
-      last = slot_of[at];
-      last_key = key;
+      last = at[h];
     }
-    uint32_t e = (uint32_t)last;
-    for (int i = 0; i < 3; i++) {
-      const int by = 1 + len + i;  // at most 10
-      const uint32_t r = (uint32_t)((by < 8 ? lo >> (8 * by) : hi >> (8 * (by - 8))) & 0xff);
-      e |= (i < rest ? r : (uint32_t)n) << (8 + 8 * i);
-    }
-    dst[(q & ~127) + 4 * (q & 31) + ((q >> 5) & 3)] = e;
+    const unsigned __int128 bytes = (unsigned __int128)hi << 64 | lo;
+    S.part.push_back(make_uint2((unsigned)last, (unsigned)(bytes >> (8 * (1 + len))) << 8));
   }
+  for (const uint64_t key : keys) S.desc.push_back(make_uint2((unsigned)key, (unsigned)(key >> 32)));
+  S.slot.assign(keys.size(), -1);
+  return S;
+}
+
+// One zone of an order's compact form: entries from `q` on as a prefix slot
+// and last ranks, slots assigned in order of first use, until another slot
+// would be needed, a prefix does not fit its descriptor, or the entries kept
+// end.  The zone stops at a whole group of four chunks.  `grp` .. `end` are the
+// order's groups, `from` the first pattern of each group in its stream.
+// Writes query 128 g + 32 c + j as lane j's c-th entry of group g; returns the
+// zone's end.
+int compact_zone(const uint2 *grp, const uint2 *end, const int64_t *from, int q, int count,
+                 std::vector<SplitStream> &split, int max_slots, uint2 *slots, uint32_t *dst) {
+  const int start = q;
+  std::pair<int, unsigned> used[sg::FAST_SLOTS];  // weight and prefix of each slot
+  int n_used = 0;
+  for (; grp < end && q < count; grp++, from++) {
+    const int first = (int)grp->x, next = grp + 1 < end ? std::min((int)grp[1].x, count) : count;
+    if (q >= next) continue;
+    const int w = (int)(grp->y >> 16);
+    SplitStream &S = split[w];
+    if (S.part.empty()) break;
+    for (; q < next; q++) {
+      const uint2 part = S.part[*from + (q - first)];  // in range: a pattern comes no later in its stream than in an order
+      int slot = S.slot[part.x];
+      if (slot < 0) {
+        if (n_used == max_slots) break;
+        slot = n_used++;
+        used[slot] = {w, part.x};
+        slots[slot] = S.desc[part.x];
+        S.slot[part.x] = (int16_t)slot;
+      }
+      dst[(q & ~127) + 4 * (q & 31) + ((q >> 5) & 3)] = (uint32_t)slot | part.y;
+    }
+    if (q < next) break;
+  }
+  for (int i = 0; i < n_used; i++) split[used[i].first].slot[used[i].second] = -1;
   return start + ((q - start) & ~127);
 }
 
@@ -224,13 +257,19 @@ int build_tables(int n, int64_t cap, int c_max, bool even, HostTables &T) {
   T.class_size = nb >= 31 ? INT32_MAX : (1 << nb);
   T.base.assign((size_t)(c_max + 1) * ncls, 0);
   T.count.assign((size_t)(c_max + 1) * ncls, 0);
+  // every order's groups and size first, then the entries: with room for all of
+  // them they are laid down once and never moved (n = 64 at cap 10^5: 31 ms
+  // instead of 57)
   int maxcost = 0, maxm = 0;
+  size_t total = 0;
+  std::vector<int64_t> from;       // first pattern of each group in its stream
+  std::vector<int> head(wtop, 0);  // patterns of each stream that an order's head may hold
   for (int c = 0; c <= c_max; c++) {
     for (int K = 0; K < ncls; K++) {
-      const size_t start = T.ent.size();
+      const size_t start = total;
       T.gbase.push_back((int32_t)T.grp.size());
       const int64_t Ctop = (int64_t)c * n + (int64_t)n * (n + 1) / 2;
-      for (int64_t C = 0; C <= Ctop && (int64_t)(T.ent.size() - start) < cap; C++) {
+      for (int64_t C = 0; C <= Ctop && (int64_t)(total - start) < cap; C++) {
         for (int w = 0; w < wtop; w++) {
           if (even && (w & 1) != K) continue;
           const int64_t m = C - (int64_t)c * w;
@@ -241,48 +280,54 @@ int build_tables(int n, int64_t cap, int c_max, bool even, HostTables &T) {
           const int64_t a = loff[w][li], b = loff[w][li + 1];
           if (b == a) continue;
           if (C > 65535) return SOGRAND_EUNSUPPORTED;
-          T.grp.push_back(make_uint2((unsigned)(T.ent.size() - start), (unsigned)m | ((unsigned)w << 16)));
+          T.grp.push_back(make_uint2((unsigned)(total - start), (unsigned)m | ((unsigned)w << 16)));
+          from.push_back(a);
+          if (total - start < sg::FAST_QUERIES)
+            head[w] = std::max(head[w], (int)std::min<int64_t>(b, sg::FAST_QUERIES));
           maxm = std::max(maxm, (int)m);
-          T.ent.insert(T.ent.end(), stream[w].begin() + a, stream[w].begin() + b);
-          T.cost.insert(T.cost.end(), (size_t)(b - a), (uint16_t)C);
           maxcost = std::max(maxcost, (int)C);
+          total += (size_t)(b - a);
         }
-        if (T.ent.size() >= (size_t(1) << 30)) return SOGRAND_ENOMEM;
+        if (total >= (size_t(1) << 30)) return SOGRAND_ENOMEM;
       }
       T.base[(size_t)c * ncls + K] = (int32_t)start;
-      T.count[(size_t)c * ncls + K] = (int32_t)(T.ent.size() - start);
+      T.count[(size_t)c * ncls + K] = (int32_t)(total - start);
     }
   }
-  // the compact forms of every order's head, built by a few threads (a
-  // million entries for n = 64: 20 ms on one)
+  T.gbase.push_back((int32_t)T.grp.size());
+  T.ent.reserve(total);
+  T.cost.reserve(total);
+  // and the compact form of each order's head, from the weights' patterns split
+  // once (splitting every order's entries anew took 6 ms more for n = 64 at cap
+  // 10^4, of 10.5 on one core; now 4.4)
   const int orders = (c_max + 1) * ncls, per = sg::FAST_SLOTS2 + sg::FAST_SLOTS;
   T.slots.assign((size_t)orders * per, make_uint2(0, 0));
   T.zones.assign(orders, make_int2(0, 0));
   const int most = std::min(*std::max_element(T.count.begin(), T.count.end()), sg::FAST_QUERIES);
   T.e4_stride = (most + 127) / 128 * 32 + 64;  // padded: two groups past the head are read ahead
   T.e4.assign((size_t)orders * T.e4_stride, make_uint4(0u, 0u, 0u, 0u));
-  std::atomic<int> next{0};
-  const auto work = [&]() {
-    for (int ti = next++; ti < orders; ti = next++) {
-      const uint4 *ent = T.ent.data() + T.base[ti];
-      const int count = std::min(T.count[ti], sg::FAST_QUERIES);
-      uint2 *slots = &T.slots[(size_t)ti * per];
-      uint32_t *dst = &T.e4[(size_t)ti * T.e4_stride].x;
-      int2 &z = T.zones[ti];
-      z.x = compact_zone(ent, 0, count, n, 2, sg::FAST_SLOTS2, slots, dst);
-      z.y = compact_zone(ent, z.x, count, n, 3, sg::FAST_SLOTS, slots + sg::FAST_SLOTS2, dst);
-    }
-  };
-  std::vector<std::thread> helpers;
-  helpers.reserve(7);
-  try {
-    for (unsigned i = 1; i < std::min(8u, std::thread::hardware_concurrency()); i++) helpers.emplace_back(work);
-  } catch (const std::exception &) {  // no more threads (or no memory for one): this thread does the rest
+  std::vector<SplitStream> split2, split3;
+  for (int w = 0; w < wtop; w++) {
+    split2.push_back(split_stream(stream[w], head[w], w, 2));
+    split3.push_back(split_stream(stream[w], head[w], w, 3));
   }
-  work();
-  for (std::thread &t : helpers) t.join();
+  for (int ti = 0; ti < orders; ti++) {
+    const int g0 = T.gbase[ti], g1 = T.gbase[ti + 1];
+    for (int g = g0; g < g1; g++) {
+      const int w = (int)(T.grp[g].y >> 16), m = (int)(T.grp[g].y & 0xffffu);
+      const int64_t a = from[g], b = a + ((g + 1 < g1 ? (int)T.grp[g + 1].x : T.count[ti]) - (int)T.grp[g].x);
+      T.ent.insert(T.ent.end(), stream[w].begin() + a, stream[w].begin() + b);
+      T.cost.insert(T.cost.end(), (size_t)(b - a), (uint16_t)(m + ti / ncls * w));
+    }
+    const int count = std::min(T.count[ti], sg::FAST_QUERIES);
+    uint2 *slots = &T.slots[(size_t)ti * per];
+    uint32_t *dst = &T.e4[(size_t)ti * T.e4_stride].x;
+    int2 &z = T.zones[ti];
+    z.x = compact_zone(&T.grp[g0], &T.grp[0] + g1, &from[g0], 0, count, split2, sg::FAST_SLOTS2, slots, dst);
+    z.y = compact_zone(&T.grp[g0], &T.grp[0] + g1, &from[g0], z.x, count, split3, sg::FAST_SLOTS,
+                       slots + sg::FAST_SLOTS2, dst);
+  }
   T.jmax = maxcost + 2;
-  T.gbase.push_back((int32_t)T.grp.size());
   // scnt[N][w][m]: w-subsets of {1..N} with sum m (N = 0..n, w < sc_w, m <= the
   // largest group sum), saturated at INT32_MAX: unranking only subtracts a
   // count smaller than the index it reduces, which is below the group's size
@@ -839,7 +884,7 @@ int persistent_check(const sogrand_code *rc_, const sogrand_code *cc_, int64_t F
   if (prc != SOGRAND_OK) return prc;
   for (const sogrand_code *x : {rc_, cc_})
     if (x->n - 1 < 63 && cap >= (int64_t(1) << (x->n - 1))) return SOGRAND_EINVAL;
-  // word tickets (slots x the larger n, plus one per idle warp) are 32-bit
+  // word tickets (slots x the larger n, plus a run of up to eight per idle warp) are 32-bit
   if (F * 2 * (int64_t)max_iter * std::max(rc_->n, cc_->n) >= (int64_t(1) << 31) - (int64_t(1) << 22))
     return SOGRAND_EINVAL;
   return SOGRAND_OK;
