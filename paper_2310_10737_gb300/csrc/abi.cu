@@ -349,38 +349,37 @@ int build_tables(int n, int64_t cap, int c_max, bool even, HostTables &T) {
   return SOGRAND_OK;
 }
 
+// One device allocation.  The three large arrays are copied from where they
+// were built, the small ones through one buffer: every copy costs the caller
+// about 10 us.
 int upload_tables(sogrand_code *c, const HostTables &T, int64_t cap) {
-  auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
-  const size_t be = T.ent.size() * sizeof(uint4), bc = T.cost.size() * sizeof(uint16_t);
-  const size_t bi = T.base.size() * sizeof(int32_t);
-  const size_t bg = T.grp.size() * sizeof(uint2), bgb = T.gbase.size() * sizeof(int32_t);
-  const size_t bs = T.scnt.size() * sizeof(int32_t);
-  const size_t b4 = T.e4.size() * sizeof(uint4), bsl = T.slots.size() * sizeof(uint2);
-  const size_t bz = T.zones.size() * sizeof(int2);
-  const size_t bytes = al(be) + al(bc) + 2 * al(bi) + al(bg) + al(bgb) + al(bs) + al(b4) + al(bsl) + al(bz);
-  void *mem = nullptr;
-  if (cudaMalloc(&mem, bytes) != cudaSuccess) return SOGRAND_ENOMEM;
-  char *p = (char *)mem;
-  uint4 *dent = (uint4 *)p;
-  uint16_t *dcost = (uint16_t *)(p + al(be));
-  int32_t *dbase = (int32_t *)(p + al(be) + al(bc));
-  int32_t *dcount = (int32_t *)(p + al(be) + al(bc) + al(bi));
-  uint2 *dgrp = (uint2 *)(p + al(be) + al(bc) + 2 * al(bi));
-  int32_t *dgbase = (int32_t *)((char *)dgrp + al(bg));
-  int32_t *dscnt = (int32_t *)((char *)dgbase + al(bgb));
-  uint4 *de4 = (uint4 *)((char *)dscnt + al(bs));
-  uint2 *dslots = (uint2 *)((char *)de4 + al(b4));
-  int2 *dzones = (int2 *)((char *)dslots + al(bsl));
-  if (cudaMemcpy(de4, T.e4.data(), b4, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dslots, T.slots.data(), bsl, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dzones, T.zones.data(), bz, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dgrp, T.grp.data(), bg, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dgbase, T.gbase.data(), bgb, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dscnt, T.scnt.data(), bs, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dent, T.ent.data(), be, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dcost, T.cost.data(), bc, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dbase, T.base.data(), bi, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(dcount, T.count.data(), bi, cudaMemcpyHostToDevice) != cudaSuccess) {
+  size_t bytes = 0;
+  const auto place = [&bytes](size_t size) {
+    const size_t at = bytes;
+    bytes += (size + 255) & ~size_t(255);
+    return at;
+  };
+  const auto size_of = [](const auto &v) { return v.size() * sizeof(v[0]); };
+  const size_t ent = place(size_of(T.ent)), cost = place(size_of(T.cost)), e4 = place(size_of(T.e4));
+  const size_t small = bytes;
+  const size_t base = place(size_of(T.base)), count = place(size_of(T.count)), grp = place(size_of(T.grp)),
+               gbase = place(size_of(T.gbase)), scnt = place(size_of(T.scnt)), slots = place(size_of(T.slots)),
+               zones = place(size_of(T.zones));
+  std::vector<char> buf(bytes - small);
+  const auto put = [&](size_t at, const auto &v) { std::memcpy(buf.data() + (at - small), v.data(), size_of(v)); };
+  put(base, T.base);
+  put(count, T.count);
+  put(grp, T.grp);
+  put(gbase, T.gbase);
+  put(scnt, T.scnt);
+  put(slots, T.slots);
+  put(zones, T.zones);
+  char *mem = nullptr;
+  if (cudaMalloc((void **)&mem, bytes) != cudaSuccess) return SOGRAND_ENOMEM;
+  if (cudaMemcpy(mem + ent, T.ent.data(), size_of(T.ent), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(mem + cost, T.cost.data(), size_of(T.cost), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(mem + e4, T.e4.data(), size_of(T.e4), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(mem + small, buf.data(), buf.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
     cudaFree(mem);
     return SOGRAND_ECUDA;
   }
@@ -389,19 +388,19 @@ int upload_tables(sogrand_code *c, const HostTables &T, int64_t cap) {
     cudaFree(c->d_tab);
   }
   c->d_tab = mem;
-  c->ord.ent = dent;
-  c->ord.cost = dcost;
-  c->ord.base = dbase;
-  c->ord.count = dcount;
+  c->ord.ent = (uint4 *)(mem + ent);
+  c->ord.cost = (uint16_t *)(mem + cost);
+  c->ord.base = (int32_t *)(mem + base);
+  c->ord.count = (int32_t *)(mem + count);
   c->ord.ncls = T.ncls;
   c->ord.class_size = T.class_size;
-  c->ord.e4 = de4;
-  c->ord.slots = dslots;
-  c->ord.zones = dzones;
+  c->ord.e4 = (uint4 *)(mem + e4);
+  c->ord.slots = (uint2 *)(mem + slots);
+  c->ord.zones = (int2 *)(mem + zones);
   c->ord.e4_stride = T.e4_stride;
-  c->grp.grp = dgrp;
-  c->grp.gbase = dgbase;
-  c->grp.scnt = dscnt;
+  c->grp.grp = (uint2 *)(mem + grp);
+  c->grp.gbase = (int32_t *)(mem + gbase);
+  c->grp.scnt = (int32_t *)(mem + scnt);
   c->grp.sc_w = T.sc_w;
   c->grp.sc_m = T.sc_m;
   c->jmax = T.jmax;
@@ -413,14 +412,12 @@ int upload_tables(sogrand_code *c, const HostTables &T, int64_t cap) {
 int reserve_locked(sogrand_code *c, int64_t cap) {
   if (cap <= c->tab_cap) return SOGRAND_OK;
   HostTables T;
-  int rc;
   try {
-    rc = build_tables(c->n, cap, c->c_max, c->even != 0, T);
+    const int rc = build_tables(c->n, cap, c->c_max, c->even != 0, T);
+    return rc == SOGRAND_OK ? upload_tables(c, T, cap) : rc;
   } catch (const std::bad_alloc &) {
     return SOGRAND_ENOMEM;
   }
-  if (rc != SOGRAND_OK) return rc;
-  return upload_tables(c, T, cap);
 }
 
 sg::DevCode dev_code(const sogrand_code *c) {
