@@ -271,8 +271,8 @@ int gldpc_decode(sogrand_code *code, int64_t n_frames, const float *llr_ch, int 
  * 128 threads per SM, 64 registers a thread) or 12 (the schedule of more
  * warps: 56 registers a thread, 9 resident blocks).  Which is faster depends
  * on the code (register pressure of its syndrome width and list against the
- * latency the extra warps hide) and is measured by sogrand_code_tune.  The default until tuned: 12 for
- * n <= 64, else 8.
+ * latency the extra warps hide) and is measured by sogrand_code_tune.  The
+ * default until tuned: 12 for n <= 64, else 8.
  *   minb     0 (query only), 8 or 12
  *   current  HOST out (may be NULL): the schedule in force
  * Not to be changed while a decode of this code is in flight.  Errors: EINVAL.

@@ -1072,7 +1072,7 @@ int sogrand_code_tune(sogrand_code *c, int64_t F, const float *llr_ch, int L, in
   const size_t nb = ((size_t)c->n * c->n + 7) / 8;
   char *bits = nullptr;
   if (scratch_alloc(&bits, al256((size_t)F * nb), s) != cudaSuccess) return SOGRAND_ENOMEM;
-  // every (blocks per SM, remaining-mass area) pair
+  // every (schedule, remaining-mass area) pair
   const int cand[4] = {8, 8, 12, 12}, cdp[4] = {0, 1, 0, 1};
   float best = 0.f, ms[2] = {0.f, 0.f};
   int pick = c->minb, pick_dp = c->dp_global;

@@ -476,7 +476,6 @@ __global__ void __launch_bounds__(TPB, resident_blocks(MINB))
   extern __shared__ __align__(16) unsigned char smem[];
   using LY = Layout<NPL, SYN>;
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const int jm = max(rowc.jmax, colc.jmax);
   unsigned char *tl = block_tail(smem, LY::warp_bytes);
   init_block_lock(tl, P);
   Scratch<NPL, SYN> sc;
@@ -657,9 +656,8 @@ __device__ __forceinline__ void frame_after_half(const DevCode &wc, const DevCod
 // bounded (a.max_spin * a.run microseconds of accumulated sleep without progress):
 // the kernel then records an error and every warp returns.  GEN: two codes or
 // wrapped diagonals (the code of a word is chosen per half); otherwise a
-// square product code whose words all use rowc, with no per-word selection
-// of a code (selecting one of two parameter structs at run time makes the
-// compiler copy it to local memory).
+// square product code whose words all use rowc, with no selection of a code
+// and its geometry in every word.
 template <int NPL, class SYN, int MINB, bool GEN, int MODE>
 __global__ void __launch_bounds__(TPB, resident_blocks(MINB))
     k_product_persistent(const __grid_constant__ DevCode rowc, const __grid_constant__ DevCode colc,
@@ -667,7 +665,6 @@ __global__ void __launch_bounds__(TPB, resident_blocks(MINB))
   extern __shared__ __align__(16) unsigned char smem[];
   using LY = Layout<NPL, SYN>;
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const int jm = max(rowc.jmax, colc.jmax);
   unsigned char *tl = block_tail(smem, LY::warp_bytes);
   init_block_lock(tl, P);
   Scratch<NPL, SYN> sc;

@@ -54,9 +54,7 @@ constexpr int FAST_QUERIES = 16384;  // most queries of an order kept in these f
 // The same orders as groups, for lanes that enumerate their patterns instead
 // of reading DevOrder::ent (DevCode::ord_lanes): a group is the run of
 // patterns of one cost and one Hamming weight w, i.e. the w-subsets of the
-// ranks {1..n} with rank sum m = cost - c w, in lexicographic order.  (A
-// struct apart from DevOrder, which the kernels copy to local memory when
-// they pass it to out-of-line functions.)
+// ranks {1..n} with rank sum m = cost - c w, in lexicographic order.
 struct DevGroups {
   const uint2 *grp;       // [groups] x: first entry of the group within its order; y: m | w << 16
   const int32_t *gbase;   // [(c_max+1) * ncls + 1] first group of order (c, class)
