@@ -40,16 +40,23 @@ L_LIST, CAP, ALPHA, MAX_ITER, SEED = 4, 10**4, 0.5, 20, 2310
 SMS, INT32_LANES = 152, 128  # GB300: 152 SMs x 128 INT32/FP32 lanes per SM
 METRIC = "decoded info bits/s, eBCH(64,57)^2 product code"
 
-# DRAM bytes (read + write) per frame of k_product_persistent, from one ncu
-# capture of a 10,000-frame decode of this workload (traffic grows with the
-# frame count at a fixed Eb/N0 mix), valid only for the kernel sources whose
-# digest is recorded with it: `traffic` is null once they change.
-TRAFFIC = {"csrc_digest": "6b1ef70c505c020836c562534333b42ff7f533e0e933b568a6ad7a3aa30e4441",
-           "bytes_per_frame": 256552.3,
+# DRAM bytes (read + write) per frame of k_product_persistent and its pipe
+# activity, from ncu captures of a 10,000-frame decode of this workload (traffic
+# grows with the frame count at a fixed Eb/N0 mix), one for each schedule: its
+# kernels are compiled apart.  Valid only for the kernel sources whose digest is
+# recorded with them and the remaining-mass area they ran with: `traffic` is
+# null otherwise.
+TRAFFIC = {"csrc_digest": "c86164ae3e53f5a765616138859e63dc7abbbb991b57efd7432fe2b50f777166",
            "source": "profiles/k_product_persistent_ebch64_57sq_10k_frames.md",
-           # pipe activity of the same capture (percent of peak sustained over active cycles)
-           "ncu": {"issue_active_pct": 75.4, "alu_pipe_pct": 50.1, "fma_pipe_pct": 32.9,
-                   "tensor_pipe_pct": 0.0, "dram_throughput_pct": 2.7}}
+           "remaining_mass_area": "shared",
+           # percent of peak sustained: issue over elapsed, pipes over active cycles
+           "schedules": {8: {"bytes_per_frame": 256457.9,
+                             "ncu": {"issue_active_pct": 76.3, "alu_pipe_pct": 49.4, "fma_pipe_pct": 32.5,
+                                     "tensor_pipe_pct": 0.0, "dram_throughput_pct": 2.6}},
+                         12: {"bytes_per_frame": 256176.6,
+                              "ncu": {"issue_active_pct": 78.7, "alu_pipe_pct": 51.8, "fma_pipe_pct": 34.0,
+                                      "tensor_pipe_pct": 0.0, "dram_throughput_pct": 2.7}}}}
+SCHEDULE_BLOCKS = {8: 8, 12: 9}  # resident blocks per SM that a schedule's kernels are compiled for
 
 
 KERNEL_SOURCES = ("kernels.cuh", "launch.h", "sg_common.h", "siso_warp.cuh")  # what k_product_persistent compiles from
@@ -509,6 +516,8 @@ def main():
     ap.add_argument("--serve-requests", type=int, default=1200, help="requests per offered load in the serving run (0: off)")
     ap.add_argument("--serve-loads", default="250,500,1000,2000,3000", help="offered loads, requests/s")
     ap.add_argument("--other-configs", type=int, default=1, help="1: also measure the C1, C2 and C4 workloads")
+    ap.add_argument("--schedule", type=int, default=0, choices=[0, 8, 12],
+                    help="schedule of the kernels (0: tuned on a sample; 8 or 12: that one, the area as the code has it)")
     ap.add_argument("--order-source", default="table", choices=["table", "lanes"],
                     help="query order of the headline decode: read from the order table, or enumerated by the lanes")
     args = ap.parse_args()
@@ -542,9 +551,12 @@ def main():
     c = sg.Code.from_linear_code(code)
     c.order_source(1 if args.order_source == "lanes" else 0)
     log("inputs resident on the device, code tables built")
-    # schedule autotuner (set-up, outside the timed region): blocks per SM on a 10,000-frame sample
-    sched, sched_ms = c.tune(d_in[: min(F, 10_000)], L=L_LIST, query_cap=CAP, alpha=ALPHA, max_iter=MAX_ITER)
-    log(f"schedule: {sched} blocks/SM (sample ms at 8 / 12: {sched_ms[0]:.1f} / {sched_ms[1]:.1f})")
+    # schedule autotuner (set-up, outside the timed region) on a 10,000-frame sample
+    sched, sched_ms = c.schedule(args.schedule), (None, None)
+    if not args.schedule:
+        sched, sched_ms = c.tune(d_in[: min(F, 10_000)], L=L_LIST, query_cap=CAP, alpha=ALPHA, max_iter=MAX_ITER)
+        log(f"schedule: {sched} (sample ms in 8 / 12: {sched_ms[0]:.1f} / {sched_ms[1]:.1f})")
+    area = "global" if c.dp_area() else "shared"
     n, k = code.n, code.k
     out = dict(bits=torch.empty((F, n * n // 8), dtype=torch.uint8, device=dev),
                half_iters=torch.empty(F, dtype=torch.int32, device=dev),
@@ -623,10 +635,13 @@ def main():
     peak = int_peak / 1e12
     achieved = ops / (t_half / 1000) / 1e12 if t_half > 0 else 0.0
     traffic = None
-    # the recorded capture is of the order-table kernel
-    same_kernel = main_persistent and args.order_source == "table" and TRAFFIC["csrc_digest"] == csrc_digest()
-    if same_kernel:
-        traffic = TRAFFIC["bytes_per_frame"] * F
+    # the recorded captures are of the order-table kernels
+    capture = None
+    if (main_persistent and args.order_source == "table" and area == TRAFFIC["remaining_mass_area"]
+            and TRAFFIC["csrc_digest"] == csrc_digest()):
+        capture = TRAFFIC["schedules"].get(sched)
+    if capture is not None:
+        traffic = capture["bytes_per_frame"] * F
     # HBM side: the LLRs in and decided bits out (algorithmic) and, from the capture, DRAM bytes
     t_launch_s = t_half / 1000 / max(half_launches, 1)
     llr_bytes = F * (4 * n * n + n * n // 8)
@@ -646,7 +661,7 @@ def main():
                             f"{int_ms:.1f} ms kernel); nominal 152 SMs x 128 lanes x {sm_max:.0f} MHz = "
                             f"{nominal:.2f} Tops/s",
                 "hbm": hbm,
-                "ncu": dict(TRAFFIC["ncu"], source=TRAFFIC["source"]) if same_kernel else None}
+                "ncu": dict(capture["ncu"], source=TRAFFIC["source"]) if capture is not None else None}
 
     # end to end through the C ABI on host buffers (copies inside the timed region)
     hout = dict(bits=torch.empty((F, n * n // 8), dtype=torch.uint8, pin_memory=True),
@@ -711,8 +726,8 @@ def main():
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "clocks": clk, "gpu_launches": launches,
                 "queries_per_s": world * qtot / (ms / 1000), "xf_words": int(out["xf_words"].item()),
                 "quality": quality, "serving": serving, "other_configs": others,
-                "schedule": {"blocks_per_sm": sched, "remaining_mass_area": ("global" if c.dp_area() else "shared"),
-                             "tuned_on": f"{min(F, 10_000)} frames",
+                "schedule": {"name": sched, "blocks_per_sm": SCHEDULE_BLOCKS[sched], "remaining_mass_area": area,
+                             "tuned_on": f"{min(F, 10_000)} frames" if not args.schedule else None,
                              "sample_ms": {"8": sched_ms[0], "12": sched_ms[1]}},
                 "form": ("persistent (one kernel per decode, device-side frame queue)" if main_persistent
                          else "plain (one launch per half iteration)"),
