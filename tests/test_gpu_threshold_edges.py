@@ -3,8 +3,10 @@ safe and the accurate functions have to decide."""
 import numpy as np
 import pytest
 
+from gpu_common import compare_siso
 from test_gpu_mass_rounding import words
 from workloads import ebch
+from workloads.codes import LinearCode
 
 pytestmark = pytest.mark.gpu
 
@@ -57,3 +59,24 @@ def test_denormal_thresholds(env, oracle_lib, name, thr):
     assert (ref["queries"] == 1).all() == (thr > 1e-38)
     np.testing.assert_array_equal(out["queries"].cpu().numpy(), ref["queries"])
     np.testing.assert_array_equal(out["list_count"].cpu().numpy(), ref["list_count"])
+
+
+@pytest.mark.parametrize("thr", [1e-11, 1e-13])
+def test_rule_with_64_bit_syndromes(env, oracle_lib, thr):
+    """40 checks (7 of them independent, so that lists fill): the rule is asked
+    at every listed word and the search goes on from the middle of a chunk of
+    16-byte entries."""
+    torch, sg = env
+    base = ebch("ebch_64_57")
+    rng = np.random.default_rng(6)
+    H = np.concatenate([base.H, (rng.integers(0, 2, (33, 7)) @ base.H % 2).astype(np.uint8)])
+    lc = LinearCode("ebch_64_57_40_checks", 64, 24, base.G, H)
+    x = rng.standard_normal((60, 64)) * rng.choice([0.5, 2.0, 6.0], (60, 1)) + rng.choice([-3.0, 0.0, 3.0], (60, 1))
+    x = x.astype(np.float32)
+    c = sg.Code.from_linear_code(lc)
+    out = sg.sogrand_decode(c, torch.from_numpy(x).cuda(), L=8, query_cap=3000, thr=thr)
+    torch.cuda.synchronize()
+    c.close()
+    ref = oracle_lib.siso_batch(oracle_lib.OracleCode(lc), x, L=8, cap=3000, thr=float(np.float32(thr)))
+    assert ref["list_count"].max() == 8
+    compare_siso(lc, out, ref, f"40 checks thr={thr}")
