@@ -548,9 +548,9 @@ __device__ __forceinline__ void dp_ranks(int Cs, int c, int R0, int cls, const t
         const T a = he[j], b = ho[j];
         T term;
         if (cls == 0)
-          term = Ops::add(Ops::mul(a, fe), Ops::mul(b, fo));
+          term = Ops::fma(a, fe, Ops::mul(b, fo));
         else if (cls == 1)
-          term = Ops::add(Ops::mul(a, fo), Ops::mul(b, fe));
+          term = Ops::fma(a, fo, Ops::mul(b, fe));
         else
           term = Ops::mul(Ops::add(a, b), Ops::add(fo, fe));
         acc = Ops::fma(w, term, acc);
