@@ -46,15 +46,15 @@ METRIC = "decoded info bits/s, eBCH(64,57)^2 product code"
 # kernels are compiled apart.  Valid only for the kernel sources whose digest is
 # recorded with them and the remaining-mass area they ran with: `traffic` is
 # null otherwise.
-TRAFFIC = {"csrc_digest": "c86164ae3e53f5a765616138859e63dc7abbbb991b57efd7432fe2b50f777166",
+TRAFFIC = {"csrc_digest": "491a570fef120c036d82b4a60c65620009652e99b2d3c2f64cda05c014b5a73e",
            "source": "profiles/k_product_persistent_ebch64_57sq_10k_frames.md",
            "remaining_mass_area": "shared",
            # percent of peak sustained: issue over elapsed, pipes over active cycles
-           "schedules": {8: {"bytes_per_frame": 256457.9,
-                             "ncu": {"issue_active_pct": 76.3, "alu_pipe_pct": 49.4, "fma_pipe_pct": 32.5,
-                                     "tensor_pipe_pct": 0.0, "dram_throughput_pct": 2.6}},
-                         12: {"bytes_per_frame": 256176.6,
-                              "ncu": {"issue_active_pct": 78.7, "alu_pipe_pct": 51.8, "fma_pipe_pct": 34.0,
+           "schedules": {8: {"bytes_per_frame": 256417.4,
+                             "ncu": {"issue_active_pct": 75.7, "alu_pipe_pct": 48.5, "fma_pipe_pct": 31.8,
+                                     "tensor_pipe_pct": 0.0, "dram_throughput_pct": 2.7}},
+                         12: {"bytes_per_frame": 256111.3,
+                              "ncu": {"issue_active_pct": 77.5, "alu_pipe_pct": 50.8, "fma_pipe_pct": 33.4,
                                       "tensor_pipe_pct": 0.0, "dram_throughput_pct": 2.7}}}}
 SCHEDULE_BLOCKS = {8: 8, 12: 9}  # resident blocks per SM that a schedule's kernels are compiled for
 
